@@ -288,6 +288,41 @@ template <typename T>
 cudaError_t launch_pack_pass(int kind, const HssLoop2<T>* plans, const int* starts, int nm, int total, int level,
                              int it, const int* live, size_t smem, cudaStream_t s);
 
+// ---- whole cycles and HSS loops of small 2D problems, one cluster each (resident.cu) ----
+// V(2,2) scaled-Jacobi cycles on `levels` levels, every level vector in distributed shared memory
+// (lv: its offsets); levels from `dist` on are held whole by every CTA.
+constexpr int kResMaxLevels = 6;
+struct ResLevel {
+    int nn, W, offA, offB, offb, offt, offr, offp;
+};
+template <typename T> struct ResArgs {
+    // filled by resident_plan
+    ResLevel lv[kResMaxLevels];
+    int levels, dist, cs, nb, elems, off_r;
+    size_t smem;
+    int dir[4];
+    // filled by the caller: coefficient records of A_L (level l, problem b at l * nb + b) and of the
+    // HSS step's A_R on level 0; sweeps on the coarsest level; HSS steps and activity flags per problem
+    const PCoef<T>* al;
+    const PCoef<T>* ar;
+    int nu_coarse;
+    const int* nhss;
+    const int* active;
+    int* status;  // set to HH_ERR_TIMEOUT when a wait ran past spin_limit polls
+    unsigned long long spin_limit;
+    const double2* r;  // HSS loop: input and result, and a vector of the problem for r in T
+    double2* z;
+    vec2<T>* r_lo;
+    const vec2<T>* b;  // one cycle: right side and result
+    vec2<T>* x;
+};
+// Fill P for nb problems on levels lv[0..levels) (hss: the HSS loop, else one cycle); false when
+// they do not fit.  Configures the kernels: call before any stream capture.
+template <typename T>
+bool resident_plan(ResArgs<T>* P, const GridDesc* lv, int levels, int nb, bool hss);
+template <typename T>
+cudaError_t launch_resident(const ResArgs<T>& P, bool hss, cudaStream_t s);
+
 // ---- GMRES smoother with a Jacobi preconditioner (gsmooth.cu) ----
 // Level vectors of nb problems (problem b at offset b * N); the Krylov basis holds vector i
 // of problem b at V + i * ld + b * N.  Sums in FP64 over a fixed block grid (gs_blocks(N)), so

@@ -20,6 +20,7 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "hh.h"
@@ -132,6 +133,10 @@ struct Hier {
     int loop_ctas = 0;
     size_t loop_smem = 0;
     bool loop_unfit = false;  // its grid does not fit the device: separate kernels instead
+    // the cluster-resident forms (hh::ResArgs<T> of this precision; [0] one cycle, [1] the HSS
+    // loop): 0 not planned yet, 1 planned, -1 not used for this problem
+    int res_state[2] = {0, 0};
+    std::vector<unsigned char> res[2];
 };
 
 }  // namespace
@@ -1087,6 +1092,60 @@ hh_status launch_loop(hh_problem* p, int prec, bool* used) {
     return HH_OK;
 }
 
+// Whether the cycles may run as one cluster-resident kernel (resident.cu): 2D primal problems with
+// the default V(2,2) scaled-Jacobi cycle, one per HSS step, and no option that asks for a form of
+// the separate kernels.
+bool resident_options(const hh_problem* p) {
+    const hh_options& o = p->o;
+    if (p->grid.dim != 2 || p->mixed || o.smoother != HH_SMOOTH_JACOBI || o.cycle_gamma != 1) return false;
+    if (o.cycles_per_hss != 1 || o.nu_pre != 2 || o.nu_post != 2 || o.nu_coarse < 1 || o.levels < 2) return false;
+    if (o.persistent != 0 || o.coarse_kernel != 0 || o.fuse_sweeps == 0 || o.tile_rows != 0 || o.tile_form != 0)
+        return false;
+    return p->lv[o.levels - 1].N <= o.coarse_cluster_nodes;
+}
+
+// The resident plan of precision T (hss: of the HSS loop, else of one cycle), or nullptr.
+template <typename T>
+hh::ResArgs<T>* resident(hh_problem* p, bool hss) {
+    Hier& H = p->hier[sizeof(T) == 4 ? HH_C64 : HH_C128];
+    if (H.res_state[hss] == 0) {
+        H.res_state[hss] = -1;
+        hh::ResArgs<T> P{};
+        // measured against the separate kernels (a V-cycle of the HSS loop / alone, us, 4 levels):
+        // complex64 17^2 9 / 17 against 35 / 41, 129^2 18 / 28 against 32 / 41, 257^2 30 / 42 against
+        // 35 / 43; complex128 33^2 34 / 42 against 136 / 128, 129^2 112 / 121 against 129 / 124
+        const long long most = sizeof(T) == 4 ? (hss ? 67000 : 40000) : (hss ? 17000 : 5000);
+        if (resident_options(p) && p->lv[0].N <= most &&
+            hh::resident_plan<T>(&P, p->lv.data(), p->o.levels, p->nb, hss)) {
+            const PCoef<T>* pc = (const PCoef<T>*)H.pc;
+            P.al = pc + (size_t)R_AL * p->o.levels * p->nb;
+            P.ar = pc + (size_t)R_AR * p->o.levels * p->nb;
+            P.nu_coarse = p->o.nu_coarse;
+            P.nhss = p->d_nhss;
+            P.active = active_flags(p);
+            P.status = (int*)(p->d_sync + 1);
+            P.spin_limit = 4194304ULL;  // (sync_spin_limit is the persistent loop's)
+            H.res[hss].resize(sizeof(P));
+            std::memcpy(H.res[hss].data(), &P, sizeof(P));
+            H.res_state[hss] = 1;
+        }
+    }
+    return H.res_state[hss] == 1 ? reinterpret_cast<hh::ResArgs<T>*>(H.res[hss].data()) : nullptr;
+}
+
+template <typename T>
+hh_status resident_hss(hh_problem* p, const double2* r, double2* z, bool* used) {
+    *used = false;
+    if (hh::ResArgs<T>* P = resident<T>(p, true)) {
+        P->r = r;
+        P->z = z;
+        P->r_lo = (hh::vec2<T>*)p->hier[sizeof(T) == 4 ? HH_C64 : HH_C128].r_lo;
+        HH_LAUNCH(hh::launch_resident<T>(*P, true, p->s));
+        *used = true;
+    }
+    return HH_OK;
+}
+
 // z (c128, nb x N) = shifted-HSS preconditioner of r (c128), on the problem stream, for the
 // active problems.
 hh_status precondition_async(hh_problem* p, const double2* r, double2* z) {
@@ -1095,6 +1154,9 @@ hh_status precondition_async(hh_problem* p, const double2* r, double2* z) {
     Hier& H = p->hier[prec];
     const long long N = p->lv[0].N;
     const long long NT = p->N * p->nb;  // (sigma and) nodes
+    bool resident_done = false;
+    HH_TRY(prec == HH_C64 ? resident_hss<float>(p, r, z, &resident_done) : resident_hss<double>(p, r, z, &resident_done));
+    if (resident_done) return HH_OK;
     if (prec == HH_C64) {
         HH_LAUNCH(hh::launch_cast_d2f(r, (float2*)H.r_lo, NT, p->s));
     } else {
@@ -1740,6 +1802,7 @@ enum PackState {
 struct PackMember {
     hh_problem* p = nullptr;
     int state = PK_FREE;
+    bool own = false;  // its preconditioner is one cluster-resident kernel on its own stream
     int io = 0;  // 0: device load vector in / device u out; 1: host load vector; 2: host nodal source
     void* u = nullptr;
     double tol = 0.0;
@@ -1786,6 +1849,7 @@ int pass_tiles(const hh::HssLoop2<float>& P, const hh_problem* p, int kind, int 
 
 hh_status enqueue_fetch(hh_problem* p) {
     HH_CUDA(cudaMemcpyAsync(p->h_host, p->hbuf, (size_t)hstride(p) * sizeof(double2), cudaMemcpyDeviceToHost, p->s));
+    HH_CUDA(cudaMemcpyAsync(p->h_sync, p->d_sync + 1, sizeof(int), cudaMemcpyDeviceToHost, p->s));
     return HH_OK;
 }
 
@@ -1933,7 +1997,7 @@ hh_status pack_rebuild(hh_pack* k) {
     k->maxsteps = 0;
     for (int i = 0; i < cap; ++i) {
         PackMember& x = k->m[i];
-        const bool in = x.state != PK_FREE && x.state != PK_DONE;
+        const bool in = x.state != PK_FREE && x.state != PK_DONE && !x.own;
         if (in) {
             MG<float> mg = make_mg<float>(x.p, HH_C64, x.p->s);
             mg.loop_plan(&plans[i]);
@@ -1994,7 +2058,7 @@ hh_status pack_round(hh_pack* k) {
     for (int i = 0; i < cap; ++i) {
         PackMember& x = k->m[i];
         k->h_live[i] = 0;
-        if (x.state != PK_NEED_ITER) continue;
+        if (x.state != PK_NEED_ITER || x.own) continue;
         hh_problem* p = x.p;
         Hier& H = p->hier[HH_C64];
         HH_LAUNCH(hh::launch_cast_d2f(p->V + (long long)x.j * p->N, (float2*)H.r_lo, p->N, p->s));
@@ -2014,10 +2078,14 @@ hh_status pack_round(hh_pack* k) {
         hh_problem* p = x.p;
         Hier& H = p->hier[HH_C64];
         const int m = p->o.restart, nrm = 2 * (m + 1);
-        HH_CUDA(cudaStreamWaitEvent(p->s, k->ev_prec, 0));
         double2* zj = p->Z + (long long)x.j * p->N;
         double2* w = p->V + (long long)(x.j + 1) * p->N;
-        HH_LAUNCH(hh::launch_gather_c128<float>((const float2* const*)H.usrc, zj, p->lv[0].N, 1, nullptr, p->s));
+        if (x.own) {
+            HH_TRY(precondition_async(p, p->V + (long long)x.j * p->N, zj));
+        } else {
+            HH_CUDA(cudaStreamWaitEvent(p->s, k->ev_prec, 0));
+            HH_LAUNCH(hh::launch_gather_c128<float>((const float2* const*)H.usrc, zj, p->lv[0].N, 1, nullptr, p->s));
+        }
         x.info.hss_its += p->nhss[0];
         x.info.vcycles += p->nhss[0];
         HH_TRY(apply_B(p, zj, w));
@@ -2034,18 +2102,26 @@ hh_status pack_round(hh_pack* k) {
         x.state = PK_ITER;
     }
     if (any) HH_CUDA(cudaStreamSynchronize(k->s));
-    for (int i = 0; i < cap; ++i) {
-        PackMember& x = k->m[i];
-        if (x.state == PK_FREE || x.state == PK_DONE) continue;
-        cudaError_t e = cudaStreamSynchronize(x.p->s);
-        if (e != cudaSuccess) {
-            pack_fail(x, fail(HH_ERR_CUDA, cudaGetErrorString(e)));
-            k->dirty = true;
-            continue;
+    // every member of the packed launches advances, and each member with launches of its own that is
+    // done (they do not wait for one another: their HSS loops differ in length); at least one does
+    bool advanced = false, waiting = true;
+    while (!advanced && waiting) {
+        waiting = false;
+        for (int i = 0; i < cap; ++i) {
+            PackMember& x = k->m[i];
+            if (x.state == PK_FREE || x.state == PK_DONE) continue;
+            const cudaError_t e = x.own ? cudaStreamQuery(x.p->s) : cudaStreamSynchronize(x.p->s);
+            if (e == cudaErrorNotReady) {
+                waiting = true;
+                continue;
+            }
+            advanced = true;
+            hh_status st = e != cudaSuccess ? fail(HH_ERR_CUDA, cudaGetErrorString(e)) : check_sync(x.p);
+            if (st == HH_OK) st = pack_after_sync(x);
+            if (st != HH_OK) pack_fail(x, st);
+            if (x.state == PK_DONE) k->dirty = true;
         }
-        const hh_status st = pack_after_sync(x);
-        if (st != HH_OK) pack_fail(x, st);
-        if (x.state == PK_DONE) k->dirty = true;
+        if (!advanced && waiting) std::this_thread::yield();
     }
     return HH_OK;
 }
@@ -2424,11 +2500,23 @@ hh_status hh_vcycle(hh_problem* p, int precision, const void* b, void* x) {
     HH_TRY(join_in(p));
     const size_t nbytes = (size_t)p->nb * p->N * (precision == HH_C64 ? 8 : 16);
     if (precision == HH_C64) {
+        if (hh::ResArgs<float>* P = resident<float>(p, false)) {
+            P->b = (const float2*)b;
+            P->x = (float2*)x;
+            HH_LAUNCH(hh::launch_resident<float>(*P, false, p->s));
+            return join_out(p);
+        }
         MG<float> m = make_mg<float>(p, precision, p->s);
         float2* out;
         HH_TRY(m.vcycle(0, (const float2*)b, nullptr, &out));
         HH_CUDA(cudaMemcpyAsync(x, out, nbytes, cudaMemcpyDeviceToDevice, p->s));
     } else {
+        if (hh::ResArgs<double>* P = resident<double>(p, false)) {
+            P->b = (const double2*)b;
+            P->x = (double2*)x;
+            HH_LAUNCH(hh::launch_resident<double>(*P, false, p->s));
+            return join_out(p);
+        }
         MG<double> m = make_mg<double>(p, precision, p->s);
         double2* out;
         HH_TRY(m.vcycle(0, (const double2*)b, nullptr, &out));
@@ -2601,6 +2689,7 @@ hh_status hh_pack_add(hh_pack* k, hh_problem* p, const void* rhs, int io, double
     PackMember& x = k->m[i];
     x = PackMember{};
     x.p = p;
+    x.own = resident<float>(p, true) != nullptr;
     x.io = io;
     x.u = u;
     x.tol = tol;
