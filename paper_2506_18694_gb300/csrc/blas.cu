@@ -44,6 +44,13 @@ __global__ void __launch_bounds__(kRedThreads) k_multidot_partial(const double2*
     w += (long long)b * kb.bs_w;
     double2 acc = make_double2(0.0, 0.0);
     const long long stride = (long long)gridDim.x * blockDim.x;
+    // a slice beyond the vector sums to 0 without a reduction: a vector of 1089 fills 5 of the 304
+    // blocks, and the FP64 adds of the others' reductions were most of the kernel's time (18.6 us for 9
+    // vectors; the 33^2 complex128 solve takes 16.2 ms without them, 17.6 with)
+    if (blockIdx.x * (long long)blockDim.x >= N) {
+        if (threadIdx.x == 0) partials[((long long)b * gridDim.y + vi) * gridDim.x + blockIdx.x] = acc;
+        return;
+    }
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += stride) {
         const double2 a = v[p], c = w[p];
         acc.x = fma(a.x, c.x, fma(a.y, c.y, acc.x));
