@@ -532,13 +532,19 @@ struct MG {
             a.y = (V2*)H->t[l];
             a.alpha = Cx<T>{-1, 0};
             a.beta = Cx<T>{1, 0};
-            HH_LAUNCH(hh::launch_march3<T>(hh::M_AXPBY, a, s));
+            HH_LAUNCH(march(hh::M_AXPBY, a));
             HH_LAUNCH(hh::launch_restrict<T>(p->lv[l + 1], (const V2*)H->t[l], rc, batch(l), s));
         }
         return HH_OK;
     }
     // xout = x~ + omega D^{-1} (b - A_L x~), x~ = x + P ec
     hh_status prolong_jacobi(int l, V2* x, const V2* ec, const V2* b, V2* xout) {
+        if (!d2()) {
+            // 3D: the correction in a pass of its own (12 thread instructions per node; interpolated on the
+            // tiles' halos in the sweep it cost more than the sweep: 306 against 115 us on 257^3)
+            HH_LAUNCH(hh::launch_prolong<T>(p->lv[l], ec, x, batch(l), s));
+            return jacobi(l, b, x, xout);
+        }
         hh::MArgs<T> a = margs(l, R_AL);
         a.x = x;
         a.ec = ec;
@@ -1392,7 +1398,7 @@ hh_status autotune(hh_problem* p, int prec) {
                                        mode == hh::M_HSS_FIRST2_RR;
             if (needs_coarser && l == L - 1) continue;
             if ((mode == hh::M_RESID_RESTRICT || mode == hh::M_PROLONG_JACOBI2 || mode == hh::M_HSS_FIRST2 ||
-                 mode == hh::M_JACOBI2_ZERO_RR || mode == hh::M_HSS_FIRST2_RR) &&
+                 mode == hh::M_JACOBI2_ZERO_RR || mode == hh::M_HSS_FIRST2_RR || mode == hh::M_PROLONG_JACOBI) &&
                 p->grid.dim == 3)
                 continue;
             if ((mode == hh::M_HSS_FIRST || mode == hh::M_HSS_FIRST2 || mode == hh::M_HSS_FIRST2_RR) && l != 0) continue;

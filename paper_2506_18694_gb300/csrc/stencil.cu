@@ -137,8 +137,58 @@ __global__ void __launch_bounds__(256) k_prolong(GridDesc gf, const vec2<T>* __r
     st<T>(x, p, ld<T>(x, p) + e);
 }
 
+// 3D: a thread takes coarse node (I, J, L) and the up to eight fine nodes (2I + a, 2J + b, 2L + c), so
+// that the coarse values it needs are read once.  The terms of a node are added in k_prolong's order
+// (z, then y, then x), so the results are the same bit for bit.
+template <typename T>
+__global__ void __launch_bounds__(256) k_prolong3(GridDesc gf, const vec2<T>* __restrict__ ec, vec2<T>* __restrict__ x,
+                                                  Batch bt) {
+    pdl_entry();
+    const int n = gf.n, nn = gf.nn, nc = n / 2, nnc = nc + 1;
+    const int b = blockIdx.z / nnc, L = blockIdx.z - b * nnc;
+    const int I = blockIdx.x * 32 + (threadIdx.x & 31), J = blockIdx.y * 8 + (threadIdx.x >> 5);
+    if (I > nc || J > nc || batch_skipped(bt, b)) return;
+    x += (long long)b * bt.bs;
+    ec += (long long)b * bt.bsc;
+    auto cd = [&](int v, int s) { return (v == 0 && gf.dir[s]) || (v == nc && gf.dir[s + 1]); };
+    Cx<T> e[2][2][2];  // coarse values (0 where no basis function: Dirichlet nodes)
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int bb = 0; bb < 2; ++bb)
+#pragma unroll
+            for (int a = 0; a < 2; ++a) {
+                const int p = I + a, q = J + bb, r = L + c;
+                const bool in = p <= nc && q <= nc && r <= nc && !cd(p, 0) && !cd(q, 2) && !cd(r, 4);
+                e[c][bb][a] = in ? ld<T>(ec, ((long long)r * nnc + q) * nnc + p) : cx<T>(0, 0);
+            }
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int bb = 0; bb < 2; ++bb)
+#pragma unroll
+            for (int a = 0; a < 2; ++a) {
+                const int i = 2 * I + a, j = 2 * J + bb, l = 2 * L + c;
+                if (i > n || j > n || l > n) continue;
+                const T w = (a ? T(0.5) : T(1)) * (bb ? T(0.5) : T(1)) * (c ? T(0.5) : T(1));
+                Cx<T> s = cx<T>(0, 0);
+#pragma unroll
+                for (int cl = 0; cl <= c; ++cl)
+#pragma unroll
+                    for (int bj = 0; bj <= bb; ++bj)
+#pragma unroll
+                        for (int ai = 0; ai <= a; ++ai) s = fma_r(w, e[cl][bj][ai], s);
+                const long long p = ((long long)l * nn + j) * nn + i;
+                st<T>(x, p, node_masked(gf, i, j, l) ? cx<T>(0, 0) : ld<T>(x, p) + s);
+            }
+}
+
 template <typename T>
 cudaError_t launch_prolong(const GridDesc& gf, const vec2<T>* ec, vec2<T>* x, const Batch& bt, cudaStream_t s) {
+    if (gf.dim == 3) {
+        const int nnc = gf.n / 2 + 1;
+        return klaunch(k_prolong3<T>, dim3((nnc + 31) / 32, (nnc + 7) / 8, nnc * bt.nb), dim3(256), 0, s, 1, gf, ec, x, bt);
+    }
     dim3 blk(32, 8, 1);
     dim3 grd((gf.nn + 31) / 32, (gf.nn + 7) / 8, (gf.dim == 3 ? gf.nn : 1) * bt.nb);
     return klaunch(k_prolong<T>, grd, blk, 0, s, 1, gf, ec, x, bt);
