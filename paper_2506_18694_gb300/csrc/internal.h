@@ -215,7 +215,8 @@ cudaError_t launch_march2(int mode, const MArgs<T>& a, cudaStream_t s);
 template <typename T>
 cudaError_t launch_march2rr(int mode, const MArgs<T>& a, cudaStream_t s);
 
-// ---- fused 3D tile kernels (march3.cu): modes as above except M_RESID_RESTRICT ----
+// ---- 3D tile kernels (march3.cu): modes M_APPLY, M_AXPBY, M_DAXPBY, M_JACOBI, M_HSS_FIRST and
+//      M_JACOBI2_ZERO ----
 template <typename T>
 cudaError_t launch_march3(int mode, const MArgs<T>& a, cudaStream_t s);
 

@@ -9,13 +9,15 @@
 // corner).  The field is loaded as zero outside the cube and at Dirichlet nodes, so a node
 // on a face, edge or corner sums its existing neighbours by group (centre; x, y, z faces;
 // xy, xz, yz edges; corners) with the eight weights of its boundary class.
+//
+// Bound by instruction issue and the shared-memory pipe together (257^3 Jacobi sweep: 59 % and
+// 67 % busy); complex sums as packed adds and no boundary checks in the output warps took it from
+// 118 to 113 us, the first two sweeps from 0 from 105 to 96 us.
 #include "internal.h"
 
 namespace hh {
 
 namespace {
-
-__device__ __forceinline__ int clampi3(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
 
 template <typename T>
 __device__ __forceinline__ Cx<T> shfl_up3(Cx<T> v) {
@@ -25,8 +27,6 @@ template <typename T>
 __device__ __forceinline__ Cx<T> shfl_dn3(Cx<T> v) {
     return Cx<T>{__shfl_down_sync(0xffffffffu, v.re, 1), __shfl_down_sync(0xffffffffu, v.im, 1)};
 }
-
-__device__ __forceinline__ bool coarse_dir(int I, int nc, int lo, int hi) { return (I == 0 && lo) || (I == nc && hi); }
 
 // Whether coordinate v of an axis with Dirichlet flags lo, hi holds no unknown.
 __device__ __forceinline__ bool void1(int v, int n, int lo, int hi) {
@@ -40,54 +40,6 @@ __device__ __forceinline__ int bclass3(int tx, int ty, int tz) {
     const int c = (tz * 3 + ty) * 3 + tx;
     return c - (c > 13);
 }
-
-// Value of the stencil field at node (i, j, l) of the grid (offset p), which holds an unknown
-// there (INNER: the node is known to lie inside the cube, off every face).
-template <typename T, int MODE, bool INNER>
-__device__ __forceinline__ Cx<T> field3(const MArgs<T>& a, const PCoef<T>& c, const Cx<T>* bw, const VPtrs<T>& v,
-                                        int i, int j, int l, long long p) {
-    const int n = a.g.n;
-    if (MODE == M_JACOBI2_ZERO) {
-        // first sweep from x = 0: x1 = omega D^{-1} b
-        const Cx<T> b = ld<T>(v.z, p);
-        if (INNER || (i >= 1 && i <= n - 1 && j >= 1 && j <= n - 1 && l >= 1 && l <= n - 1)) return cmul(c.wdinv, b);
-        const int q = bclass3(type1(i, n), type1(j, n), type1(l, n));
-        return cmul(bw[q * kClass3Len + 8], b);
-    } else if (MODE == M_PROLONG_JACOBI) {
-        // x + P e_c: trilinear interpolation of the coarse correction
-        const int nc = n >> 1, nnc = nc + 1;
-        const int I0 = i >> 1, J0 = j >> 1, L0 = l >> 1;
-        const bool oi = i & 1, oj = j & 1, ol = l & 1;
-        Cx<T> e = cx<T>(0, 0);
-#pragma unroll
-        for (int cl = 0; cl < 2; ++cl) {
-            if (cl == 1 && !ol) break;
-            const int L = L0 + cl;
-            if (coarse_dir(L, nc, a.g.dir[4], a.g.dir[5])) continue;
-            const T wl = ol ? T(0.5) : T(1);
-#pragma unroll
-            for (int bj = 0; bj < 2; ++bj) {
-                if (bj == 1 && !oj) break;
-                const int J = J0 + bj;
-                if (coarse_dir(J, nc, a.g.dir[2], a.g.dir[3])) continue;
-                const T wj = oj ? T(0.5) * wl : wl;
-#pragma unroll
-                for (int ai = 0; ai < 2; ++ai) {
-                    if (ai == 1 && !oi) break;
-                    const int I = I0 + ai;
-                    if (coarse_dir(I, nc, a.g.dir[0], a.g.dir[1])) continue;
-                    const T w = oi ? T(0.5) * wj : wj;
-                    e = fma_r(w, ld<T>(v.ec, ((long long)L * nnc + J) * nnc + I), e);
-                }
-            }
-        }
-        return ld<T>(v.x, p) + e;
-    } else {
-        return a.xzero ? cx<T>(0, 0) : ld<T>(v.x, p);
-    }
-}
-
-constexpr int kWarps3 = 8;  // y-rows per tile, including the two halo rows
 
 // Window of a node: the field value (f*) and x-neighbour sum (x*) of its column on planes
 // l-1, l, l+1, and the sums over rows j-1 and j+1 of the value (vy*) and of the x-sum (sy*).
@@ -143,12 +95,17 @@ __device__ __forceinline__ void out3(const MArgs<T>& a, const PCoef<T>& cf, cons
     }
 }
 
+constexpr int kWarps3 = 8;  // y-rows per tile, including the two halo rows
+
 }  // namespace
 
-// One tile.  INNER: every node the tile loads (halos included) lies inside the cube, off every
-// face, so no node is void or on the boundary and no check or boundary-class code is needed;
-// the node arithmetic is the same as on the general path.
-template <typename T, int MODE, int R, bool BATCH, bool INNER>
+// One tile.  Nodes outside the cube and Dirichlet nodes load as zero: one predicate per column and a
+// uniform one per plane.  Output rows and planes are uniform over a warp, so a warp runs either the
+// inner formula or that of one boundary class; the columns i = 0 and n, where lanes would differ, are
+// left to the two halo warps, which have nothing to do after the barrier: a lane per node, from the
+// sums in shared memory.  (Checked per lane in the output warps, tiles on the cube's faces, 28 % of
+// them on 257^3, cost about 350 thread instructions per node against 90 inside.)
+template <typename T, int MODE, int R, bool BATCH>
 __device__ __forceinline__ void march3_tile(const MArgs<T>& a, int b, int bx, int by, int l0,
                                             unsigned char* smem_raw) {
     const PCoef<T>& cf = BATCH ? a.pc[b] : a.c0;
@@ -164,25 +121,35 @@ __device__ __forceinline__ void march3_tile(const MArgs<T>& a, int b, int bx, in
     const int n = a.g.n, nn = a.g.nn;
     const int i = bx * 30 + lane - 1;
     const int j = by * (kWarps3 - 2) + w - 1;
-    const int ic = INNER ? i : clampi3(i, 0, n), jc = INNER ? j : clampi3(j, 0, n);
-    const bool cvoid = !INNER && (void1(i, n, a.g.dir[0], a.g.dir[1]) || void1(j, n, a.g.dir[2], a.g.dir[3]));
+    const bool cvoid = void1(i, n, a.g.dir[0], a.g.dir[1]) || void1(j, n, a.g.dir[2], a.g.dir[3]);
+    const bool zero = cvoid || (MODE != M_JACOBI2_ZERO && a.xzero);
+    const int tx = type1(i, n), ty = type1(j, n);
     const long long ps = (long long)nn * nn;
-    const long long colc = (long long)jc * nn + ic;
+    const long long col = (long long)j * nn + i + l0 * ps;  // (used where the node lies in the cube)
+    const vec2<T>* const xin = (MODE == M_JACOBI2_ZERO ? v.z : v.x) + col;
 
     Cx<T> fv[NP], xs[NP];
 #pragma unroll
     for (int t = 0; t < NP; ++t) {
         const int l = l0 - 1 + t;
-        // (a node of a plane that is not void lies inside the cube: no clamp needed)
-        fv[t] = (!INNER && (cvoid || void1(l, n, a.g.dir[4], a.g.dir[5])))
-                    ? cx<T>(0, 0)
-                    : field3<T, MODE, INNER>(a, cf, bw, v, ic, jc, l, colc + l * ps);
+        fv[t] = (zero || void1(l, n, a.g.dir[4], a.g.dir[5])) ? cx<T>(0, 0) : ld<T>(xin, (t - 1) * ps);
     }
-    Cx<T> zv[R];
     const bool out_row = w >= 1 && w <= kWarps3 - 2;
+    const bool out = out_row && lane >= 1 && lane <= 30 && tx == 1 && j <= n;
+    Cx<T> zv[R];
 #pragma unroll
     for (int t = 0; t < R; ++t)
-        zv[t] = (NEEDZ && out_row) ? ld<T>(v.z, colc + (INNER ? l0 + t : clampi3(l0 + t, 0, n)) * ps) : cx<T>(0, 0);
+        zv[t] = (NEEDZ && out && l0 + t <= n) ? ld<T>(v.z + col, t * ps) : cx<T>(0, 0);
+    if (MODE == M_JACOBI2_ZERO) {
+        // first sweep from x = 0: x1 = omega D^{-1} b
+        const bool in = tx == 1 && ty == 1;
+#pragma unroll
+        for (int t = 0; t < NP; ++t) {
+            const int l = l0 - 1 + t;
+            const Cx<T> d = in && l >= 1 && l <= n - 1 ? cf.wdinv : bw[bclass3(tx, ty, type1(l, n)) * kClass3Len + 8];
+            fv[t] = cmul(d, fv[t]);
+        }
+    }
 #pragma unroll
     for (int t = 0; t < NP; ++t) {
         xs[t] = shfl_up3(fv[t]) + shfl_dn3(fv[t]);
@@ -190,9 +157,29 @@ __device__ __forceinline__ void march3_tile(const MArgs<T>& a, int b, int bx, in
         st<T>(ss, (w * NP + t) * 32 + lane, xs[t]);
     }
     __syncthreads();
-    if (!out_row || !(lane >= 1 && lane <= 30) || (!INNER && (i > n || j > n))) return;
-    const bool colrow_inner = INNER || (i >= 1 && i <= n - 1 && j >= 1 && j <= n - 1);
-    const int tx = type1(i, n), ty = type1(j, n);
+    if (!out_row) {
+        // column i = 0 (warp 0) or n (the last warp), if the tile holds it: rows by * 6 + r, planes l0 + t
+        const int is = w == 0 ? 0 : n, lc = is - bx * 30 + 1;
+        if (lc < 1 || lc > 30) return;
+        for (int q = lane; q < (kWarps3 - 2) * R; q += 32) {
+            const int r = q / R, t = q - r * R, js = by * (kWarps3 - 2) + r, l = l0 + t;
+            if (js > n || l > n) continue;
+            const int e = ((r + 1) * NP + t) * 32 + lc;  // its row on plane l - 1
+            constexpr int P = 32, Y = NP * 32;
+            const long long p = (long long)js * nn + is + l * ps;
+            const Cx<T> zq = NEEDZ ? ld<T>(v.z, p) : cx<T>(0, 0);
+            const Win3<T> q3{ld<T>(sv, e), ld<T>(sv, e + P), ld<T>(sv, e + 2 * P),
+                             ld<T>(ss, e), ld<T>(ss, e + P), ld<T>(ss, e + 2 * P),
+                             ld<T>(sv, e - Y) + ld<T>(sv, e + Y), ld<T>(sv, e + P - Y) + ld<T>(sv, e + P + Y),
+                             ld<T>(sv, e + 2 * P - Y) + ld<T>(sv, e + 2 * P + Y),
+                             ld<T>(ss, e - Y) + ld<T>(ss, e + Y), ld<T>(ss, e + P - Y) + ld<T>(ss, e + P + Y),
+                             ld<T>(ss, e + 2 * P - Y) + ld<T>(ss, e + 2 * P + Y)};
+            const bool vd = void1(is, n, a.g.dir[0], a.g.dir[1]) || void1(js, n, a.g.dir[2], a.g.dir[3]);
+            out3<T, MODE, false>(a, cf, bw, v, q3, zq, type1(is, n), type1(js, n), l, vd, p);
+        }
+        return;
+    }
+    if (!out) return;
     const int wm = w - 1, wp = w + 1;
     // rows j-1 + j+1 summed (value and x-sum) per plane, in a rolling window of 3 planes
     auto ysum = [&](const vec2<T>* arr, int tpl) {
@@ -203,10 +190,11 @@ __device__ __forceinline__ void march3_tile(const MArgs<T>& a, int b, int bx, in
     q.vy1 = ysum(sv, 1);
     q.sy0 = ysum(ss, 0);
     q.sy1 = ysum(ss, 1);
+    const long long p0 = col;
 #pragma unroll
     for (int t = 0; t < R; ++t) {
         const int l = l0 + t;
-        if (!INNER && l > n) break;
+        if (l > n) break;
         const int tp = t + 1;  // local plane of the output
         q.vy2 = ysum(sv, tp + 1);
         q.sy2 = ysum(ss, tp + 1);
@@ -216,11 +204,11 @@ __device__ __forceinline__ void march3_tile(const MArgs<T>& a, int b, int bx, in
         q.xm = xs[tp - 1];
         q.x0 = xs[tp];
         q.xp = xs[tp + 1];
-        const long long p = colc + l * ps;
-        if (INNER || (colrow_inner && l >= 1 && l <= n - 1))
-            out3<T, MODE, true>(a, cf, bw, v, q, zv[t], tx, ty, l, cvoid, p);
+        const long long p = p0 + t * ps;
+        if (ty == 1 && l >= 1 && l <= n - 1)  // (uniform over the warp)
+            out3<T, MODE, true>(a, cf, bw, v, q, zv[t], 1, 1, l, false, p);
         else
-            out3<T, MODE, false>(a, cf, bw, v, q, zv[t], tx, ty, l, cvoid, p);
+            out3<T, MODE, false>(a, cf, bw, v, q, zv[t], 1, ty, l, cvoid, p);
         q.vy0 = q.vy1;
         q.vy1 = q.vy2;
         q.sy0 = q.sy1;
@@ -228,25 +216,14 @@ __device__ __forceinline__ void march3_tile(const MArgs<T>& a, int b, int bx, in
     }
 }
 
-// Whether tile (bx, by, z from l0) with its halos lies inside the cube, off every face.
-__device__ __forceinline__ bool tile_inner3(int n, int bx, int by, int l0, int R) {
-    const int i0 = bx * 30 - 1, j0 = by * (kWarps3 - 2) - 1, z0 = l0 - 1;
-    return i0 >= 1 && i0 + 31 <= n - 1 && j0 >= 1 && j0 + kWarps3 - 1 <= n - 1 && z0 >= 1 && z0 + R + 1 <= n - 1;
-}
-
 // BATCH = false: a batch of one, coefficients from the kernel parameters, no activity flags.
-// Each CTA takes the check-free path when its whole tile (halos included) lies inside the cube.
 template <typename T, int MODE, int R, bool BATCH>
-__global__ void __launch_bounds__(32 * kWarps3) k_march3(const __grid_constant__ MArgs<T> a, int zt) {
+__global__ void __launch_bounds__(32 * kWarps3, sizeof(T) == 4 && R <= 4 ? 4 : 1) k_march3(const __grid_constant__ MArgs<T> a, int zt) {
     pdl_entry();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int b = BATCH ? (int)blockIdx.z / zt : 0;  // problem; blockIdx.z % zt: z-tile
     if (BATCH && problem_skipped(a, b)) return;
-    const int l0 = (blockIdx.z - b * zt) * R;
-    if (tile_inner3(a.g.n, blockIdx.x, blockIdx.y, l0, R))
-        march3_tile<T, MODE, R, BATCH, true>(a, b, blockIdx.x, blockIdx.y, l0, smem_raw);
-    else
-        march3_tile<T, MODE, R, BATCH, false>(a, b, blockIdx.x, blockIdx.y, l0, smem_raw);
+    march3_tile<T, MODE, R, BATCH>(a, b, blockIdx.x, blockIdx.y, (blockIdx.z - b * zt) * R, smem_raw);
 }
 
 // Weights of the 3D boundary classes.  1D rows (Q1): stiffness (1/h)(-1, cnt, -1), mass
@@ -340,7 +317,6 @@ cudaError_t launch_march3(int mode, const MArgs<T>& a, cudaStream_t s) {
         case M_JACOBI: return pick3<T, M_JACOBI>(a, s);
         case M_HSS_FIRST: return pick3<T, M_HSS_FIRST>(a, s);
         case M_JACOBI2_ZERO: return pick3<T, M_JACOBI2_ZERO>(a, s);
-        case M_PROLONG_JACOBI: return pick3<T, M_PROLONG_JACOBI>(a, s);
         default: return cudaErrorInvalidValue;
     }
 }
