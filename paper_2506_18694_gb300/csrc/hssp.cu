@@ -101,9 +101,7 @@ __device__ __forceinline__ void f_pass(const MArgs<T>& a, int strips, int chunks
         const PCoef<T>& c = BATCH ? a.pc[b] : a.c0;
         const PCoef<T>& cl = BATCH ? a.pc2[b] : a.c02;
         const VPtrs<T> v = problem_ptrs(a, b, false);
-        TileF<T, 2> tl;
-        tilef_load<T, M_PROLONG_JACOBI2, 2>(a, v, r % strips, r / strips, tl);
-        tilef_compute<T, M_PROLONG_JACOBI2, 2>(a, c, cl, v, r % strips, r / strips, tl);
+        tilef<T, M_PROLONG_JACOBI2, 2>(a, c, cl, v, r % strips, r / strips);
     }
 }
 

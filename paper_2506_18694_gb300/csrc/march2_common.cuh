@@ -37,6 +37,14 @@ __device__ __forceinline__ bool row_void(const MArgs<T>& a, int r) {
     return r < 0 || r > a.g.n || (r == 0 && a.g.dir[2]) || (r == a.g.n && a.g.dir[3]);
 }
 
+// Whether a tile of 32 columns from `left` and `rows` rows from `first` lies inside the grid, off its
+// sides (at least `off` nodes): no node of it is void, on a boundary or beside the grid, and the tile
+// functions compile without those checks (INNER).  Uniform over the warp.
+template <typename T>
+__device__ __forceinline__ bool tile_inner2(const MArgs<T>& a, int left, int first, int rows, int off = 1) {
+    return left >= off && left + 31 <= a.g.n - off && first >= off && first + rows - 1 <= a.g.n - off;
+}
+
 // op f at row t of a tile column (interior weights or the node's boundary class), with
 // omega D^{-1} of the record's opd.
 template <typename T>
@@ -64,25 +72,26 @@ __device__ __forceinline__ void stencil_node2(const PCoef<T>& c, Cx<T> fm, Cx<T>
 // per lane: the lane at an even fine column takes its coarse value, a lane at an odd column
 // the mean of its own and its right neighbour's (by shuffle; lane 31 reads its second value
 // itself); odd fine rows then average two interpolated coarse rows.  Coarse nodes on a
-// Dirichlet side carry no basis function and count as zero.
-template <typename T, int NR, int P>
+// Dirichlet side carry no basis function and count as zero.  INNER: the fine nodes lie at least two
+// nodes off the sides, so that every coarse node that counts is an inner one.
+template <typename T, int NR, int P, bool INNER>
 __device__ __forceinline__ void prolong_rows(const MArgs<T>& a, const VPtrs<T>& v, int ic, int rfirst, bool cvoid,
                                              Cx<T>* out) {
     const int n = a.g.n, nc = n >> 1, nnc = nc + 1;
     const int lane = threadIdx.x & 31;
     const int I = ic >> 1;
-    const int I1 = I + 1 <= nc ? I + 1 : nc;
+    const int I1 = INNER || I + 1 <= nc ? I + 1 : nc;
     const bool odd = ic & 1;
-    const bool v0 = (I == 0 && a.g.dir[0]) || (I == nc && a.g.dir[1]);
-    const bool v1 = (I1 == 0 && a.g.dir[0]) || (I1 == nc && a.g.dir[1]);
+    const bool v0 = !INNER && ((I == 0 && a.g.dir[0]) || (I == nc && a.g.dir[1]));
+    const bool v1 = !INNER && ((I1 == 0 && a.g.dir[0]) || (I1 == nc && a.g.dir[1]));
     constexpr int NCR = ((P + NR) >> 1) + 1;
     const int J0 = rfirst >> 1;  // floor(rfirst / 2)
     Cx<T> ex[NCR];
 #pragma unroll
     for (int q = 0; q < NCR; ++q) {
         const int J = J0 + q;
-        const bool jv = J < 0 || J > nc || (J == 0 && a.g.dir[2]) || (J == nc && a.g.dir[3]);
-        const long long row = (long long)clampi(J, 0, nc) * nnc;
+        const bool jv = !INNER && (J < 0 || J > nc || (J == 0 && a.g.dir[2]) || (J == nc && a.g.dir[3]));
+        const long long row = (long long)(INNER ? J : clampi(J, 0, nc)) * nnc;
         const Cx<T> c0 = (jv || v0) ? cx<T>(0, 0) : ld<T>(v.ec, row + I);
         Cx<T> c1 = shfl_dn(c0);
         if (lane == 31) c1 = (jv || v1) ? cx<T>(0, 0) : ld<T>(v.ec, row + I1);
@@ -91,10 +100,10 @@ __device__ __forceinline__ void prolong_rows(const MArgs<T>& a, const VPtrs<T>& 
 #pragma unroll
     for (int t = 0; t < NR; ++t) {
         const int r = rfirst + t;
-        const long long p = (long long)clampi(r, 0, n) * a.g.nn + ic;
+        const long long p = (long long)(INNER ? r : clampi(r, 0, n)) * a.g.nn + ic;
         const int lq = (P + t) >> 1;
         const Cx<T> e = ((P + t) & 1) == 0 ? ex[lq] : half_rn(ex[lq] + ex[lq + 1]);
-        out[t] = (cvoid || row_void(a, r)) ? cx<T>(0, 0) : ld<T>(v.x, p) + e;
+        out[t] = (!INNER && (cvoid || row_void(a, r))) ? cx<T>(0, 0) : ld<T>(v.x, p) + e;
     }
 }
 
@@ -110,7 +119,7 @@ template <typename T, int ROWS> struct TileF {
     Cx<T> zv[NR - 2];  // b (PROLONG_JACOBI2) or r (HSS_FIRST2) on rows 1..NR-2
 };
 
-template <typename T, int MODE, int ROWS>
+template <typename T, int MODE, int ROWS, bool INNER>
 __device__ __forceinline__ void tilef_load(const MArgs<T>& a, const VPtrs<T>& v, int strip, int cy,
                                            TileF<T, ROWS>& tl) {
     constexpr int NR = TileF<T, ROWS>::NR;
@@ -118,23 +127,24 @@ __device__ __forceinline__ void tilef_load(const MArgs<T>& a, const VPtrs<T>& v,
     const int n = a.g.n;
     const int i = strip * 28 + lane - 2;
     const int rfirst = cy * ROWS - 2;
-    const int ic = clampi(i, 0, n);
-    const bool cvoid = col_void(a, i);
+    const int ic = INNER ? i : clampi(i, 0, n);
+    const bool cvoid = !INNER && col_void(a, i);
     if (MODE == M_PROLONG_JACOBI2) {
-        prolong_rows<T, NR, 0>(a, v, ic, rfirst, cvoid, tl.fv);  // (first row cy * ROWS - 2 is even)
+        prolong_rows<T, NR, 0, INNER>(a, v, ic, rfirst, cvoid, tl.fv);  // (first row cy * ROWS - 2 is even)
     } else {
 #pragma unroll
         for (int t = 0; t < NR; ++t) {
             const int r = rfirst + t;
-            const long long p = (long long)clampi(r, 0, n) * a.g.nn + ic;
-            tl.fv[t] = (a.xzero || cvoid || row_void(a, r)) ? cx<T>(0, 0) : ld<T>(v.x, p);
+            const long long p = (long long)(INNER ? r : clampi(r, 0, n)) * a.g.nn + ic;
+            tl.fv[t] = (a.xzero || (!INNER && (cvoid || row_void(a, r)))) ? cx<T>(0, 0) : ld<T>(v.x, p);
         }
     }
 #pragma unroll
-    for (int t = 0; t < NR - 2; ++t) tl.zv[t] = ld<T>(v.z, (long long)clampi(rfirst + 1 + t, 0, n) * a.g.nn + ic);
+    for (int t = 0; t < NR - 2; ++t)
+        tl.zv[t] = ld<T>(v.z, (long long)(INNER ? rfirst + 1 + t : clampi(rfirst + 1 + t, 0, n)) * a.g.nn + ic);
 }
 
-template <typename T, int MODE, int ROWS>
+template <typename T, int MODE, int ROWS, bool INNER>
 __device__ __forceinline__ void tilef_compute(const MArgs<T>& a, const PCoef<T>& c, const PCoef<T>& cl,
                                               const VPtrs<T>& v, int strip, int cy, TileF<T, ROWS>& tl) {
     constexpr int NR = TileF<T, ROWS>::NR;
@@ -142,11 +152,11 @@ __device__ __forceinline__ void tilef_compute(const MArgs<T>& a, const PCoef<T>&
     const int n = a.g.n;
     const int i = strip * 28 + lane - 2;
     const int rfirst = cy * ROWS - 2;
-    const int ic = clampi(i, 0, n);
-    const bool col_in = (i >= 0 && i <= n);
-    const bool col_inner = (i >= 1 && i <= n - 1);
-    const bool cvoid = col_void(a, i);
-    const int tx = ic == 0 ? 0 : (ic == n ? 2 : 1);
+    const int ic = INNER ? i : clampi(i, 0, n);
+    const bool col_in = INNER || (i >= 0 && i <= n);
+    const bool col_inner = INNER || (i >= 1 && i <= n - 1);
+    const bool cvoid = !INNER && col_void(a, i);
+    const int tx = INNER ? 1 : (ic == 0 ? 0 : (ic == n ? 2 : 1));
     const Cx<T>* fv = tl.fv;
     Cx<T> lf[NR], rg[NR];
 #pragma unroll
@@ -161,13 +171,13 @@ __device__ __forceinline__ void tilef_compute(const MArgs<T>& a, const PCoef<T>&
 #pragma unroll
     for (int t = 1; t < NR - 1; ++t) {
         const int j = rfirst + t;
-        const int jc = clampi(j, 0, n);
-        const bool fast = col_inner && j >= 1 && j <= n - 1;
+        const int jc = INNER ? j : clampi(j, 0, n);
+        const bool fast = INNER || (col_inner && j >= 1 && j <= n - 1);
         const int ty = jc == 0 ? 0 : (jc == n ? 2 : 1);
         Cx<T> ax, dinv_w;
         stencil_node2(c, fv[t - 1], fv[t], fv[t + 1], lf[t - 1], lf[t], lf[t + 1], rg[t - 1], rg[t], rg[t + 1], fast,
                       tx, ty, ax, dinv_w);
-        const bool vd = cvoid || row_void(a, j);
+        const bool vd = !INNER && (cvoid || row_void(a, j));
         if (MODE == M_PROLONG_JACOBI2) {
             b2[t] = tl.zv[t - 1];
             x1[t] = vd ? cx<T>(0, 0) : fma_c(dinv_w, tl.zv[t - 1] - ax, fv[t]);
@@ -186,9 +196,9 @@ __device__ __forceinline__ void tilef_compute(const MArgs<T>& a, const PCoef<T>&
 #pragma unroll
     for (int t = 2; t < NR - 2; ++t) {
         const int j = rfirst + t;
-        const bool row_in = (j >= 0 && j <= n);
-        const int jc = clampi(j, 0, n);
-        const bool fast = col_inner && j >= 1 && j <= n - 1;
+        const bool row_in = INNER || (j >= 0 && j <= n);
+        const int jc = INNER ? j : clampi(j, 0, n);
+        const bool fast = INNER || (col_inner && j >= 1 && j <= n - 1);
         const int ty = jc == 0 ? 0 : (jc == n ? 2 : 1);
         Cx<T> ax, dinv_w;
         stencil_node2(cl, x1[t - 1], x1[t], x1[t + 1], lf[t - 1], lf[t], lf[t + 1], rg[t - 1], rg[t], rg[t + 1], fast,
@@ -211,6 +221,20 @@ __device__ __forceinline__ void tilef_compute(const MArgs<T>& a, const PCoef<T>&
     }
 }
 
+// One warp's tile of a fused mode.
+template <typename T, int MODE, int ROWS>
+__device__ __forceinline__ void tilef(const MArgs<T>& a, const PCoef<T>& c, const PCoef<T>& cl, const VPtrs<T>& v,
+                                      int strip, int cy) {
+    TileF<T, ROWS> tl;
+    if (tile_inner2(a, strip * 28 - 2, cy * ROWS - 2, ROWS + 4, MODE == M_PROLONG_JACOBI2 ? 2 : 1)) {
+        tilef_load<T, MODE, ROWS, true>(a, v, strip, cy, tl);
+        tilef_compute<T, MODE, ROWS, true>(a, c, cl, v, strip, cy, tl);
+    } else {
+        tilef_load<T, MODE, ROWS, false>(a, v, strip, cy, tl);
+        tilef_compute<T, MODE, ROWS, false>(a, c, cl, v, strip, cy, tl);
+    }
+}
+
 // Geometry of a mode: lane of the first output column (fine column strip * S + lane - OFF),
 // fine columns per strip, stencil rows loaded.
 template <int MODE, int CR> struct RRGeo {
@@ -223,8 +247,8 @@ template <int MODE, int CR> struct RRGeo {
 
 // One warp's tile of the pre-smoothing + residual-restriction pass: fine-column strip
 // `strip`, coarse rows cy * CR .. cy * CR + CR - 1 of problem b.
-template <typename T, int MODE, int CR, bool BATCH>
-__device__ __forceinline__ void rr_tile(const MArgs<T>& a, int b, int strip, int cy) {
+template <typename T, int MODE, int CR, bool BATCH, bool INNER>
+__device__ __forceinline__ void rr_tile_of(const MArgs<T>& a, int b, int strip, int cy) {
     using G = RRGeo<MODE, CR>;
     constexpr int NF = G::NF;
     const PCoef<T>& c = BATCH ? a.pc[b] : a.c0;    // first stage (A_R for the HSS step, else A_L)
@@ -236,20 +260,21 @@ __device__ __forceinline__ void rr_tile(const MArgs<T>& a, int b, int strip, int
     const int i = strip * G::S + lane - G::OFF;
     const int J0 = cy * CR;
     const int rfirst = 2 * J0 - 1 - G::RES0;  // fine row of tile row 0
-    const int ic = clampi(i, 0, n);
-    const bool col_in = i >= 0 && i <= n;
-    const bool col_inner = i >= 1 && i <= n - 1;
-    const bool cvoid = col_void(a, i);
-    const int tx = ic == 0 ? 0 : (ic == n ? 2 : 1);
+    const int ic = INNER ? i : clampi(i, 0, n);
+    const bool col_in = INNER || (i >= 0 && i <= n);
+    const bool col_inner = INNER || (i >= 1 && i <= n - 1);
+    const bool cvoid = !INNER && col_void(a, i);
+    const int tx = INNER ? 1 : (ic == 0 ? 0 : (ic == n ? 2 : 1));
     auto row_of = [&](int t) { return rfirst + t; };
-    auto ptr = [&](int t) { return (long long)clampi(row_of(t), 0, n) * nn + ic; };
+    auto ptr = [&](int t) { return (long long)(INNER ? row_of(t) : clampi(row_of(t), 0, n)) * nn + ic; };
+    auto rvoid = [&](int j) { return !INNER && (cvoid || row_void(a, j)); };
 
     // ---- loads: the field source on every tile row, the right side where it is used
     Cx<T> f[NF], z[NF];
 #pragma unroll
     for (int t = 0; t < NF; ++t) {
         if (G::HSS) {
-            f[t] = (a.xzero || cvoid || row_void(a, row_of(t))) ? cx<T>(0, 0) : ld<T>(v.x, ptr(t));
+            f[t] = (a.xzero || rvoid(row_of(t))) ? cx<T>(0, 0) : ld<T>(v.x, ptr(t));
             z[t] = (t >= 1 && t <= NF - 2) ? ld<T>(v.z, ptr(t)) : cx<T>(0, 0);
         } else {
             z[t] = ld<T>(v.z, ptr(t));  // b, also the source of the first sweep
@@ -269,13 +294,13 @@ __device__ __forceinline__ void rr_tile(const MArgs<T>& a, int b, int strip, int
         bb[0] = bb[NF - 1] = x1[0] = x1[NF - 1] = cx<T>(0, 0);
 #pragma unroll
         for (int t = 1; t < NF - 1; ++t) {
-            const int j = row_of(t), jc = clampi(j, 0, n);
-            const bool fast = col_inner && j >= 1 && j <= n - 1;
+            const int j = row_of(t), jc = INNER ? j : clampi(j, 0, n);
+            const bool fast = INNER || (col_inner && j >= 1 && j <= n - 1);
             const int ty = jc == 0 ? 0 : (jc == n ? 2 : 1);
             Cx<T> ax, dinv_w;
             stencil_node2(c, f[t - 1], f[t], f[t + 1], lf[t - 1], lf[t], lf[t + 1], rg[t - 1], rg[t], rg[t + 1], fast,
                           tx, ty, ax, dinv_w);
-            const bool vd = cvoid || row_void(a, j);
+            const bool vd = rvoid(j);
             const Cx<T> rhs = fma_c(alpha, ax, cmul(beta, z[t]));
             bb[t] = vd ? cx<T>(0, 0) : rhs;
             x1[t] = vd ? cx<T>(0, 0) : cmul(dinv_w, rhs);
@@ -286,9 +311,9 @@ __device__ __forceinline__ void rr_tile(const MArgs<T>& a, int b, int strip, int
         for (int t = 0; t < NF; ++t) {
             const int r = row_of(t);
             bb[t] = z[t];
-            if (cvoid || row_void(a, r)) {
+            if (rvoid(r)) {
                 x1[t] = cx<T>(0, 0);
-            } else if (col_inner && r >= 1 && r <= n - 1) {
+            } else if (INNER || (col_inner && r >= 1 && r <= n - 1)) {
                 x1[t] = cmul(cl.wdinv, z[t]);
             } else {
                 const int ty = r == 0 ? 0 : (r == n ? 2 : 1);
@@ -309,13 +334,13 @@ __device__ __forceinline__ void rr_tile(const MArgs<T>& a, int b, int strip, int
         }
 #pragma unroll
         for (int t = s2; t < NF - s2; ++t) {
-            const int j = row_of(t), jc = clampi(j, 0, n);
-            const bool fast = col_inner && j >= 1 && j <= n - 1;
+            const int j = row_of(t), jc = INNER ? j : clampi(j, 0, n);
+            const bool fast = INNER || (col_inner && j >= 1 && j <= n - 1);
             const int ty = jc == 0 ? 0 : (jc == n ? 2 : 1);
             Cx<T> ax, dinv_w;
             stencil_node2(cl, x1[t - 1], x1[t], x1[t + 1], lf[t - 1], lf[t], lf[t + 1], rg[t - 1], rg[t], rg[t + 1],
                           fast, tx, ty, ax, dinv_w);
-            const bool vd = cvoid || row_void(a, j);
+            const bool vd = rvoid(j);
             x2[t] = vd ? cx<T>(0, 0) : fma_c(dinv_w, bb[t] - ax, x1[t]);
         }
     }
@@ -324,7 +349,7 @@ __device__ __forceinline__ void rr_tile(const MArgs<T>& a, int b, int strip, int
 #pragma unroll
     for (int t = G::RES0 + 1; t < G::RES0 + 1 + 2 * CR; ++t) {
         const int j = row_of(t);
-        if (!own_col || j < 0 || j > n) continue;
+        if (!own_col || (!INNER && (j < 0 || j > n))) continue;
         const long long p = (long long)j * nn + ic;
         if (G::HSS) {
             st<T>(v.y, p, bb[t]);
@@ -344,9 +369,9 @@ __device__ __forceinline__ void rr_tile(const MArgs<T>& a, int b, int strip, int
 #pragma unroll
     for (int t = G::RES0; t <= G::RES0 + 2 * CR; ++t) {
         const int j = row_of(t);
-        const bool row_in = j >= 0 && j <= n;
-        const int jc = clampi(j, 0, n);
-        const bool fast = col_inner && j >= 1 && j <= n - 1;
+        const bool row_in = INNER || (j >= 0 && j <= n);
+        const int jc = INNER ? j : clampi(j, 0, n);
+        const bool fast = INNER || (col_inner && j >= 1 && j <= n - 1);
         const int ty = jc == 0 ? 0 : (jc == n ? 2 : 1);
         Cx<T> ax, dinv_w;
         stencil_node2(cl, x2[t - 1], x2[t], x2[t + 1], lf[t - 1], lf[t], lf[t + 1], rg[t - 1], rg[t], rg[t + 1], fast,
@@ -364,14 +389,22 @@ __device__ __forceinline__ void rr_tile(const MArgs<T>& a, int b, int strip, int
                 const int J = J0 + tl / 2 - 1;
                 const int I = strip * (G::S / 2) + ((lane - G::OFF) >> 1);
                 if (lane >= G::OFF && lane < G::OFF + G::S && !((lane - G::OFF) & 1) && I <= nc && J <= nc) {
-                    const bool cm = (I == 0 && a.g.dir[0]) || (I == nc && a.g.dir[1]) || (J == 0 && a.g.dir[2]) ||
-                                    (J == nc && a.g.dir[3]);
+                    const bool cm = !INNER && ((I == 0 && a.g.dir[0]) || (I == nc && a.g.dir[1]) || (J == 0 && a.g.dir[2]) ||
+                                    (J == nc && a.g.dir[3]));
                     st<T>(yc, (long long)J * (nc + 1) + I, cm ? cx<T>(0, 0) : acc);
                 }
             }
             acc = half_rn(rr);
         }
     }
+}
+template <typename T, int MODE, int CR, bool BATCH>
+__device__ __forceinline__ void rr_tile(const MArgs<T>& a, int b, int strip, int cy) {
+    using G = RRGeo<MODE, CR>;
+    if (tile_inner2(a, strip * G::S - G::OFF, 2 * cy * CR - 1 - G::RES0, G::NF))
+        rr_tile_of<T, MODE, CR, BATCH, true>(a, b, strip, cy);
+    else
+        rr_tile_of<T, MODE, CR, BATCH, false>(a, b, strip, cy);
 }
 
 // One scaled-Jacobi update of node pi of a padded 2D slab (row width W), with the weights of its

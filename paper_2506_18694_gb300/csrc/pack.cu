@@ -58,9 +58,7 @@ __global__ void __launch_bounds__(128) k_pack_f(const HssLoop2<T>* __restrict__ 
     const int strips = P.post_strips[level];
     const int r = t - starts[m];
     const VPtrs<T> v = problem_ptrs(a, 0, false);
-    TileF<T, 2> tl;
-    tilef_load<T, M_PROLONG_JACOBI2, 2>(a, v, r % strips, r / strips, tl);
-    tilef_compute<T, M_PROLONG_JACOBI2, 2>(a, a.c0, a.c02, v, r % strips, r / strips, tl);
+    tilef<T, M_PROLONG_JACOBI2, 2>(a, a.c0, a.c02, v, r % strips, r / strips);
 }
 
 // the coarsest level: one CTA per band of coarse_rows rows of one problem
