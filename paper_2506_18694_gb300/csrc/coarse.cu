@@ -330,6 +330,9 @@ static int g_cluster_size = 0;
 
 int coarse_cluster_size() {
     if (g_cluster_size) return g_cluster_size;
+    // the query below asks for kCoarseSmemMax, which the queried kernel has to be allowed: where only the
+    // complex128 kernels had been prepared it failed and the level ran in one CTA (33^2: 128 us)
+    cudaFuncSetAttribute(k_coarse_dsmem<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmemMax);
     cudaFuncSetAttribute(k_coarse_dsmem<float>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     cudaFuncSetAttribute(k_coarse_dsmem<double>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     cudaFuncSetAttribute(k_coarse_dsmem2<float>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
