@@ -121,10 +121,11 @@ typedef struct {
     int tile_rows;       /* rows (2D) / z-planes (3D) per warp tile of the stencil kernels:   */
                          /* 2, 4 or 8; 0 = chosen from the grid size                          */
     int autotune;        /* 1: run hh_autotune for `precision` when the problem is created    */
-    int fuse_sweeps;     /* 1: in 2D, on levels of at most 600000 nodes (all problems of a     */
-                         /* batch together), consecutive steps of the cycle run as one kernel */
-                         /* (with V(2,*): the two pre-sweeps, or the HSS right side and them, */
-                         /* with the residual restriction; the prolongation with the first    */
+    int fuse_sweeps;     /* 1: in 2D, consecutive steps of the cycle run as one kernel where that is */
+                         /* the faster form (complex64: levels of one problem, and of batches up to   */
+                         /* 600000 nodes altogether; complex128: levels of at most 3000 nodes)        */
+                         /* (with V(2,*): the two pre-sweeps, or the HSS right side and them,         */
+                         /* with the residual restriction; the prolongation with the first           */
                          /* two post-sweeps); same result bit for bit as 0 (one kernel each)  */
     int outer;           /* hh_outer: HH_OUTER_FGMRES (default) or HH_OUTER_RICHARDSON      */
     int cycle_gamma;     /* multigrid cycle index 1..4: 1 V-cycle (default), 2 W-cycle (the    */

@@ -14,6 +14,7 @@
 #include <mutex>
 #include <tuple>
 #include <chrono>
+#include <climits>
 #include <cmath>
 #include <atomic>
 #include <complex>
@@ -476,10 +477,15 @@ struct MG {
         return a;
     }
 
-    // two consecutive sweeps of level l run as one pass (2D): it removes a launch and a trip
-    // through memory but computes the first sweep on a wider halo, which pays while the
-    // level is latency-bound (measured: faster up to 513^2 nodes, slower from 1025^2)
-    bool fused2(int l) const { return d2() && p->o.fuse_sweeps && Nl(l) * p->nb <= 600000; }
+    // two consecutive sweeps of level l run as one pass (2D): it removes a launch and a trip through
+    // memory but computes the first sweep on a wider halo.  complex64: pays at every size for one problem
+    // (V-cycle on 513^2 48, on 1025^2 71 against 74, on 4097^2 444 against 473 us), and for batches while
+    // they are latency-bound (128 x 64 problems: 102 fused, 95 separate).  complex128 is bound by FP64
+    // operations, which the halos multiply (513^2: 417 us fused, 284 separate): tiny levels only.
+    bool fused2(int l) const {
+        const long long most = sizeof(T) == 8 ? 3000 : (p->nb == 1 ? LLONG_MAX : 600000);
+        return d2() && p->o.fuse_sweeps && Nl(l) * p->nb <= most;
+    }
 
     hh::Batch batch(int l) const {
         return hh::Batch{p->nb, Nl(l), l + 1 < p->o.levels ? Nl(l + 1) : 0, p->nb == 1 ? -1 : hss_it, p->d_nhss,
