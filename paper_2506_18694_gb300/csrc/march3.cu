@@ -11,8 +11,9 @@
 // xy, xz, yz edges; corners) with the eight weights of its boundary class.
 //
 // Bound by instruction issue and the shared-memory pipe together (257^3 Jacobi sweep: 59 % and
-// 67 % busy); complex sums as packed adds and no boundary checks in the output warps took it from
-// 118 to 113 us, the first two sweeps from 0 from 105 to 96 us.
+// 67 % busy).  Complex sums as packed adds and no boundary checks in the output warps took the
+// sweep from 118 to 113 us; tiles off every face (72 % of them there) compiled without any check, to
+// 109 us, and the V-cycle of that grid from 769 to 740.
 #include "internal.h"
 
 namespace hh {
@@ -103,9 +104,9 @@ constexpr int kWarps3 = 8;  // y-rows per tile, including the two halo rows
 // uniform one per plane.  Output rows and planes are uniform over a warp, so a warp runs either the
 // inner formula or that of one boundary class; the columns i = 0 and n, where lanes would differ, are
 // left to the two halo warps, which have nothing to do after the barrier: a lane per node, from the
-// sums in shared memory.  (Checked per lane in the output warps, tiles on the cube's faces, 28 % of
-// them on 257^3, cost about 350 thread instructions per node against 90 inside.)
-template <typename T, int MODE, int R, bool BATCH>
+// sums in shared memory.  INNER: every node the tile loads lies inside the cube, off every face, and
+// no check is made at all.
+template <typename T, int MODE, int R, bool BATCH, bool INNER>
 __device__ __forceinline__ void march3_tile(const MArgs<T>& a, int b, int bx, int by, int l0,
                                             unsigned char* smem_raw) {
     const PCoef<T>& cf = BATCH ? a.pc[b] : a.c0;
@@ -121,9 +122,9 @@ __device__ __forceinline__ void march3_tile(const MArgs<T>& a, int b, int bx, in
     const int n = a.g.n, nn = a.g.nn;
     const int i = bx * 30 + lane - 1;
     const int j = by * (kWarps3 - 2) + w - 1;
-    const bool cvoid = void1(i, n, a.g.dir[0], a.g.dir[1]) || void1(j, n, a.g.dir[2], a.g.dir[3]);
+    const bool cvoid = !INNER && (void1(i, n, a.g.dir[0], a.g.dir[1]) || void1(j, n, a.g.dir[2], a.g.dir[3]));
     const bool zero = cvoid || (MODE != M_JACOBI2_ZERO && a.xzero);
-    const int tx = type1(i, n), ty = type1(j, n);
+    const int tx = INNER ? 1 : type1(i, n), ty = INNER ? 1 : type1(j, n);
     const long long ps = (long long)nn * nn;
     const long long col = (long long)j * nn + i + l0 * ps;  // (used where the node lies in the cube)
     const vec2<T>* const xin = (MODE == M_JACOBI2_ZERO ? v.z : v.x) + col;
@@ -132,21 +133,21 @@ __device__ __forceinline__ void march3_tile(const MArgs<T>& a, int b, int bx, in
 #pragma unroll
     for (int t = 0; t < NP; ++t) {
         const int l = l0 - 1 + t;
-        fv[t] = (zero || void1(l, n, a.g.dir[4], a.g.dir[5])) ? cx<T>(0, 0) : ld<T>(xin, (t - 1) * ps);
+        fv[t] = (zero || (!INNER && void1(l, n, a.g.dir[4], a.g.dir[5]))) ? cx<T>(0, 0) : ld<T>(xin, (t - 1) * ps);
     }
     const bool out_row = w >= 1 && w <= kWarps3 - 2;
-    const bool out = out_row && lane >= 1 && lane <= 30 && tx == 1 && j <= n;
+    const bool out = out_row && lane >= 1 && lane <= 30 && (INNER || (tx == 1 && j <= n));
     Cx<T> zv[R];
 #pragma unroll
     for (int t = 0; t < R; ++t)
-        zv[t] = (NEEDZ && out && l0 + t <= n) ? ld<T>(v.z + col, t * ps) : cx<T>(0, 0);
+        zv[t] = (NEEDZ && out && (INNER || l0 + t <= n)) ? ld<T>(v.z + col, t * ps) : cx<T>(0, 0);
     if (MODE == M_JACOBI2_ZERO) {
         // first sweep from x = 0: x1 = omega D^{-1} b
         const bool in = tx == 1 && ty == 1;
 #pragma unroll
         for (int t = 0; t < NP; ++t) {
             const int l = l0 - 1 + t;
-            const Cx<T> d = in && l >= 1 && l <= n - 1 ? cf.wdinv : bw[bclass3(tx, ty, type1(l, n)) * kClass3Len + 8];
+            const Cx<T> d = INNER || (in && l >= 1 && l <= n - 1) ? cf.wdinv : bw[bclass3(tx, ty, type1(l, n)) * kClass3Len + 8];
             fv[t] = cmul(d, fv[t]);
         }
     }
@@ -157,6 +158,7 @@ __device__ __forceinline__ void march3_tile(const MArgs<T>& a, int b, int bx, in
         st<T>(ss, (w * NP + t) * 32 + lane, xs[t]);
     }
     __syncthreads();
+    if (INNER && !out_row) return;
     if (!out_row) {
         // column i = 0 (warp 0) or n (the last warp), if the tile holds it: rows by * 6 + r, planes l0 + t
         const int is = w == 0 ? 0 : n, lc = is - bx * 30 + 1;
@@ -194,7 +196,7 @@ __device__ __forceinline__ void march3_tile(const MArgs<T>& a, int b, int bx, in
 #pragma unroll
     for (int t = 0; t < R; ++t) {
         const int l = l0 + t;
-        if (l > n) break;
+        if (!INNER && l > n) break;
         const int tp = t + 1;  // local plane of the output
         q.vy2 = ysum(sv, tp + 1);
         q.sy2 = ysum(ss, tp + 1);
@@ -205,7 +207,7 @@ __device__ __forceinline__ void march3_tile(const MArgs<T>& a, int b, int bx, in
         q.x0 = xs[tp];
         q.xp = xs[tp + 1];
         const long long p = p0 + t * ps;
-        if (ty == 1 && l >= 1 && l <= n - 1)  // (uniform over the warp)
+        if (INNER || (ty == 1 && l >= 1 && l <= n - 1))  // (uniform over the warp)
             out3<T, MODE, true>(a, cf, bw, v, q, zv[t], 1, 1, l, false, p);
         else
             out3<T, MODE, false>(a, cf, bw, v, q, zv[t], 1, ty, l, cvoid, p);
@@ -223,7 +225,12 @@ __global__ void __launch_bounds__(32 * kWarps3, sizeof(T) == 4 && R <= 4 ? 4 : 1
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int b = BATCH ? (int)blockIdx.z / zt : 0;  // problem; blockIdx.z % zt: z-tile
     if (BATCH && problem_skipped(a, b)) return;
-    march3_tile<T, MODE, R, BATCH>(a, b, blockIdx.x, blockIdx.y, (blockIdx.z - b * zt) * R, smem_raw);
+    const int l0 = (blockIdx.z - b * zt) * R, n = a.g.n;
+    const int i0 = (int)blockIdx.x * 30 - 1, j0 = (int)blockIdx.y * (kWarps3 - 2) - 1, z0 = l0 - 1;
+    if (i0 >= 1 && i0 + 31 <= n - 1 && j0 >= 1 && j0 + kWarps3 - 1 <= n - 1 && z0 >= 1 && z0 + R + 1 <= n - 1)
+        march3_tile<T, MODE, R, BATCH, true>(a, b, blockIdx.x, blockIdx.y, l0, smem_raw);
+    else
+        march3_tile<T, MODE, R, BATCH, false>(a, b, blockIdx.x, blockIdx.y, l0, smem_raw);
 }
 
 // Weights of the 3D boundary classes.  1D rows (Q1): stiffness (1/h)(-1, cnt, -1), mass
