@@ -11,8 +11,15 @@
 // combined in FP64: each block writes its share, and the kernel that uses a sum adds the
 // shares in a fixed order (every block of that kernel the same way), so the result is the
 // same whatever ran before and however the problems are batched.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+#include <mutex>
+
 #include "internal.h"
 #include "march2_common.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace hh {
 
@@ -268,195 +275,563 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_update(vec2<T>* __restrict__ 
     }
 }
 
-// ---- the whole smoothing step in one CTA per problem (small 2D levels) ----
-constexpr int kGsCtaThreads = 1024;
+// ---- the whole smoothing step in one launch: a cluster per problem ----
+// Why.  A step of 5 iterations as separate kernels is 34 launches of 3 to 4 us, and in one CTA with the
+// basis in global memory it took 85 us on 65^2.  Here (GB300, complex64, 5 iterations) a step takes
+// 12 us on 9^2, 18 on 33^2, 24 on 65^2, 33 on 129^2 and 62 on 257^2; the W-cycle of 257^2 went from 2372 to
+// 712 us, of 129^2 from 1535 to 531, complex128 129^2 from 9428 to 3400.  A small level is bound by the
+// chain of two sums an iteration (500 cycles in a block, 1350 more for the cluster barrier),
+// 257^2 by the shared-memory reads of the basis (four times an iteration).
+//
+// The Krylov basis of a level lives in the (distributed) shared memory of the cluster, a band of
+// rows per CTA with a halo row above and below and a zero column beside the row; w stays in
+// registers.  What is left of an iteration is two sums over the cluster, each one cluster barrier.
+// The halo rows of w travel with the first; the receiver makes the next basis vector's halo rows
+// of them as the sender does its own rows.  The norm comes from the second pass' sums: with c the
+// coefficients of that pass and w before it, h^2 = ||w||^2 - ||c||^2, exact to rounding while ||c||^2 is
+// a small part of ||w||^2; else (w almost in the space already) it is summed by itself.
+//
+// Sums: a thread's and a warp's in the level precision; over the warps and the CTAs as pairs of
+// a sum and its rounding error (complex64), in a fixed order.
+#ifndef GSNT
+#define GSNT 1024
+#define GSKN 5
+#endif
+template <typename T> struct GsCfg;  // threads a CTA at most
+template <> struct GsCfg<float> {
+    static constexpr int kThreads = 1024;
+};
+template <> struct GsCfg<double> {
+    static constexpr int kThreads = 512;
+};
+constexpr int kGsScal = 2 * kGsMaxIts + 1;  // scalars of a sum
+// A level takes the fewest CTAs that leave one no more nodes than this (halo rows included), if 16 are
+// enough.  W-cycle of 257^2 with GMRES(5), us, for 300, 512, 1024, 2048, 4096 nodes: 756, 751, 785, 793, 932;
+// 32 problems of 129^2 together 1281, 1210, 1196, 959, 911; complex128 129^2 3184, 3441, 3827, 4542, 5674.
+constexpr int kGsBand = 512;
+constexpr int kGsClusterMax = 16;  // (non-portable; fewer where the device does not hold one)
+constexpr size_t kGsSmemMax = 226 * 1024;
 
-// sum over the block of every thread's acc[i] (i < nv) into out[i] (shared), fixed order
-template <typename T>
-__device__ void cta_sums(Cx<T> (&acc)[kGsMaxVec], int nv, Cx<T> (*red)[kGsMaxVec], Cx<T>* out) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int i = 0; i < kGsMaxVec; ++i) {
-        if (i >= nv) break;
-        Cx<T> v = acc[i];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            v.re += __shfl_xor_sync(0xffffffffu, v.re, o);
-            v.im += __shfl_xor_sync(0xffffffffu, v.im, o);
-        }
-        if (lane == 0) red[wid][i] = v;
+template <typename T> struct Sum;
+template <> struct Sum<float> {
+    float hi, lo;
+    __device__ static Sum of(float v) { return Sum{v, 0.0f}; }
+    // (an infinite or NaN sum makes its rounding error NaN: the sum alone counts then)
+    __device__ float value() const { return lo == lo ? hi + lo : hi; }
+    __device__ Sum plus_lane(int o) const {
+        const float h2 = __shfl_xor_sync(0xffffffffu, hi, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
+        const float t = __fadd_rn(hi, h2), bb = __fsub_rn(t, hi);
+        const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(t, bb)), __fsub_rn(h2, bb));
+        return Sum{t, __fadd_rn(__fadd_rn(lo, l2), err)};
     }
+};
+template <> struct Sum<double> {
+    double hi;
+    __device__ static Sum of(double v) { return Sum{v}; }
+    __device__ double value() const { return hi; }
+    __device__ Sum plus_lane(int o) const { return Sum{hi + __shfl_xor_sync(0xffffffffu, hi, o)}; }
+};
+
+// Weights of a node's kind (boundary class 0..7, 8 inner): centre, x, y and diagonal neighbours,
+// omega D^{-1}.
+template <typename T> struct alignas(4 * sizeof(T)) GsWeights {
+    Cx<T> w[4], dinv, pad;
+};
+
+// Start of the dynamic shared memory; the basis vectors follow at kGsHead<T> bytes.
+template <typename T> struct GsShared {
+    GsWeights<T> wt[9];
+    T red[32][kGsScal + 2];  // sums of the warps (a group of sums may end beyond the last vector's)
+    Sum<T> part[2][kGsClusterMax][kGsScal];
+    T H[kGsMaxIts][2][kGsScal];  // the sums of column j: both passes' coefficients; ||w||^2
+    T beta2, tmp, h[kGsMaxIts];
+    Cx<T> R[kGsMaxIts][kGsMaxIts];
+    Cx<T> g[kGsMaxVec], sn[kGsMaxIts], ys[kGsMaxIts];
+    T cs[kGsMaxIts];
+};
+template <typename T> constexpr size_t kGsHead = (sizeof(GsShared<T>) + 127) / 128 * 128;
+
+// A node word: offset in a basis vector, kind, flags (up, dn: sent to that neighbour; free: holds an
+// unknown; in: own row, else a halo row).  0: no node; offset 0 is an entry that stays 0.
+constexpr unsigned kGsUp = 1u << 20, kGsDn = 1u << 21, kGsFree = 1u << 22, kGsIn = 1u << 23, kGsHalo = 1u << 24;
+constexpr unsigned kGsInner = 1u << 25;  // every lane of the warp has an inner node there
+
+template <typename T> struct GsCtx {
+    GsShared<T>* sh;
+    vec2<T>*vup, *vdn;  // the neighbours' V, shifted so that a sent row's offset is that of their halo row
+    vec2<T>* V;         // basis vector i at V + i * ss, row r of the band at (r + 1) * W, column i at + i + 1
+    int W, ss, R, rank, cs, phase;
+};
+
+// v[0..S) summed over the warp: 32 / S lanes end with each sum; to red[0..S)
+template <typename T, int S>
+__device__ __forceinline__ void warp_sums(T* v, T* red) {
+    const int lane = threadIdx.x & 31;
+    int o = 16;
+#pragma unroll
+    for (int h = S / 2; h >= 1; h >>= 1, o >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const T keep = up ? v[i + h] : v[i], give = up ? v[i] : v[i + h];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+#pragma unroll
+    for (; o >= 1; o >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    if ((lane & (32 / S - 1)) == 0) red[lane / (32 / S)] = v[0];
+}
+
+// Column `col` of H, from both passes' sums and the norm h below its diagonal: the previous
+// rotations, then the one that zeroes h; the right side g with it.
+template <typename T>
+__device__ __forceinline__ void rotate_column(GsShared<T>& s, int col) {
+    auto H = [&](int i) {
+        return cx<T>(s.H[col][0][2 * i] + s.H[col][1][2 * i], s.H[col][0][2 * i + 1] + s.H[col][1][2 * i + 1]);
+    };
+    Cx<T> a = H(0);
+    for (int i = 0; i < col; ++i) {
+        Cx<T> q = H(i + 1);
+        rotate<T>(s.cs[i], s.sn[i], a, q);
+        s.R[i][col] = a;
+        a = q;
+    }
+    const T h = s.h[col];
+    const T a2 = a.re * a.re + a.im * a.im, na = sqrt(a2), den = sqrt(a2 + h * h);
+    T c = T(1);
+    Cx<T> sn = cx<T>(0, 0);
+    if (den > T(0)) {
+        if (na == T(0)) {
+            c = T(0);
+            sn = cx<T>(1, 0);
+        } else {
+            // s = (a / |a|) h / den (H's entries are of the order of 1: nothing overflows)
+            const T q = h / (na * den);
+            c = na / den;
+            sn = cx<T>(a.re * q, a.im * q);
+        }
+    }
+    s.cs[col] = c;
+    s.sn[col] = sn;
+    s.R[col][col] = cx<T>(c * a.re + sn.re * h, c * a.im + sn.im * h);
+    const Cx<T> g0 = s.g[col];
+    s.g[col] = cx<T>(c * g0.re, c * g0.im);
+    s.g[col + 1] = cx<T>(-(sn.re * g0.re + sn.im * g0.im), -(sn.re * g0.im - sn.im * g0.re));
+}
+
+// Back substitution R y = g by one warp, row i by lane i; a zero pivot (breakdown: the space was
+// already invariant) gives y_j = 0.
+template <typename T>
+__device__ __forceinline__ void back_substitute(GsShared<T>& s, int its) {
+    const int i = threadIdx.x & 31, r = min(i, its - 1);
+    Cx<T> t = s.g[r];
+    const Cx<T> p = s.R[r][r];
+    const T dd = p.re * p.re + p.im * p.im;
+    const Cx<T> inv = dd > T(0) ? cx<T>(p.re / dd, -p.im / dd) : cx<T>(0, 0);
+    for (int j = its - 1; j >= 0; --j) {
+        Cx<T> y = cmul(t, inv);
+        y = cx<T>(__shfl_sync(0xffffffffu, y.re, j), __shfl_sync(0xffffffffu, y.im, j));
+        if (i == j) s.ys[j] = y;
+        if (i < j) t = t - cmul(s.R[i][j], y);
+    }
+}
+
+// The warps' sums red[.][0..ns) over the cluster into out, the same in every CTA.  rot >= 0: meanwhile
+// the last warp reduces column rot by rotations.
+template <typename T>
+__device__ __forceinline__ void cluster_sums(GsCtx<T>& x, int ns, T* out, int rot = -1) {
+    const int nw = blockDim.x >> 5, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    GsShared<T>& sh = *x.sh;
     __syncthreads();
-    if ((int)threadIdx.x < nv) {
-        Cx<T> t = cx<T>(0, 0);
-        for (int w = 0; w < kGsCtaThreads / 32; ++w) t = t + red[w][threadIdx.x];
-        out[threadIdx.x] = t;
+    Sum<T>(*part)[kGsScal] = sh.part[x.phase & 1];
+    for (int q = wid; q < ns; q += nw) {
+        Sum<T> t = Sum<T>::of(lane < nw ? sh.red[lane][q] : T(0));
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) t = t.plus_lane(o);  // (every lane ends with the sum)
+        if (x.cs == 1) {
+            if (lane == 0) out[q] = t.value();
+        } else if (lane < x.cs) {
+            *cg::this_cluster().map_shared_rank(&part[x.rank][q], lane) = t;
+        }
+    }
+    if (rot >= 0 && threadIdx.x == blockDim.x - 32) rotate_column<T>(sh, rot);
+    if (x.cs > 1) {
+        __syncwarp();
+        cg::this_cluster().sync();
+        for (int q = wid; q < ns; q += nw) {
+            Sum<T> t = lane < x.cs ? part[lane][q] : Sum<T>::of(T(0));
+            for (int o = x.cs >> 1; o >= 1; o >>= 1) t = t.plus_lane(o);
+            if (lane == 0) out[q] = t.value();
+        }
+        ++x.phase;
     }
     __syncthreads();
 }
 
-// grid (nb): problem blockIdx.x.  x (in/out), b, and the basis V_0..V_its (+ work vector
-// V_{its+1}) at Vb + i * ldv, all with problem offsets b * N.
+// op f at a node of a zero-padded band, and omega D^{-1} of the node
 template <typename T>
-__global__ void __launch_bounds__(kGsCtaThreads) k_gs_cta(const __grid_constant__ MArgs<T> a,
-                                                          const vec2<T>* __restrict__ bvec, vec2<T>* x, int xzero,
-                                                          int its, vec2<T>* Vb, long long ldv) {
-    pdl_entry();
-    const int pb = blockIdx.x;
-    if (a.pc && problem_skipped(a, pb)) return;  // the whole CTA
-    const PCoef<T>& c = a.pc ? a.pc[pb] : a.c0;
-    const int n = a.g.n, nn = a.g.nn;
-    const long long N = a.g.N;
-    const long long off = (long long)pb * N;
-    const vec2<T>* bb = bvec + off;
-    vec2<T>* xb = x + off;
-    auto V = [&](int i) { return Vb + (long long)i * ldv + off; };
-    vec2<T>* W = V(its + 1);
-    __shared__ Cx<T> red[kGsCtaThreads / 32][kGsMaxVec];
-    __shared__ Cx<T> hc[kGsMaxVec];
-    __shared__ Cx<T> R[kGsMaxVec][kGsMaxIts];
-    __shared__ Cx<T> g[kGsMaxVec], sn[kGsMaxIts], ys[kGsMaxIts];
-    __shared__ T csv[kGsMaxIts];
-    __shared__ T scal;
-    auto dirn = [&](int i, int j) {
+__device__ __forceinline__ Cx<T> band_apply(const GsWeights<T>* wt, const vec2<T>* f, int W, unsigned d, Cx<T>* dinv) {
+    const vec2<T>* p = f + (d & 0xffff);
+    const GsWeights<T>& k = wt[d & kGsInner ? 8 : (d >> 16) & 15];
+    const Cx<T> hx = ld<T>(p, -1) + ld<T>(p, 1), vy = ld<T>(p, -W) + ld<T>(p, W);
+    const Cx<T> dg = (ld<T>(p, -W - 1) + ld<T>(p, -W + 1)) + (ld<T>(p, W - 1) + ld<T>(p, W + 1));
+    *dinv = k.dinv;
+    if (d & kGsInner) {  // (fewer shared loads: 257^2 spends its time on them)
+        const GsWeights<T>& c = wt[8];
+        return fma_c(c.w[3], dg, fma_c(c.w[1], hx + vy, cmul(c.w[0], ld<T>(p, 0))));
+    }
+    return fma_c(k.w[3], dg, fma_c(k.w[2], vy, fma_c(k.w[1], hx, cmul(k.w[0], ld<T>(p, 0)))));
+}
+
+// w to the neighbours' halo rows of basis vector `to`, and (after a sum) from there
+template <typename T, int KN>
+__device__ __forceinline__ void send_rows(const GsCtx<T>& x, const unsigned* d, const Cx<T>* w, int to) {
+    if (x.cs == 1) return;
+#pragma unroll
+    for (int k = 0; k < KN; ++k) {
+        if (d[k] & kGsUp) st<T>(x.vup, to * x.ss + (d[k] & 0xffff), w[k]);
+        if (d[k] & kGsDn) st<T>(x.vdn, to * x.ss + (d[k] & 0xffff), w[k]);
+    }
+}
+template <typename T, int KN>
+__device__ __forceinline__ void take_rows(const GsCtx<T>& x, const unsigned* d, Cx<T>* w, int from) {
+    if (x.cs == 1) return;
+#pragma unroll
+    for (int k = 0; k < KN; ++k)
+        if (d[k] & kGsHalo) w[k] = ld<T>(x.V, from * x.ss + (d[k] & 0xffff));
+}
+
+// the warp's share of ||w||^2 on the own rows, as scalar q of the sums
+template <typename T, int KN>
+__device__ __forceinline__ void norm_share(const GsCtx<T>& x, const unsigned* d, const Cx<T>* w, int q) {
+    T acc = T(0);
+#pragma unroll
+    for (int k = 0; k < KN; ++k) {
+        const Cx<T> u = d[k] & kGsIn ? w[k] : cx<T>(0, 0);
+        acc = fmaT(u.re, u.re, fmaT(u.im, u.im, acc));
+    }
+    __syncwarp();  // (a group of sums may have written there)
+    warp_sums<T, 1>(&acc, &x.sh->red[threadIdx.x >> 5][q]);
+}
+
+// w orthogonalised against v_0..v_{nv-1} by classical Gram-Schmidt, twice: column nv - 1 of H; its
+// squared norm the return value.  Straight-line over a thread's KN nodes (those it has not read an
+// entry that is 0), in groups of kGroup vectors.
+template <typename T, int KN>
+__device__ __forceinline__ T orthogonalise(GsCtx<T>& x, const unsigned* d, Cx<T>* w, int nv, bool more) {
+    constexpr int kGroup = 4;
+    GsShared<T>& sh = *x.sh;
+    T(*H)[kGsScal] = sh.H[nv - 1];
+    if (more) send_rows<T, KN>(x, d, w, nv);
+    T sq = T(0);
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+        const vec2<T>* v0 = x.V;
+#pragma unroll 1
+        for (int i0 = 0; i0 < nv; i0 += kGroup, v0 += kGroup * x.ss) {
+            T acc[2 * kGroup];
+#pragma unroll
+            for (int i = 0; i < 2 * kGroup; ++i) acc[i] = T(0);
+#pragma unroll
+            for (int k = 0; k < KN; ++k) {
+                const vec2<T>* p = v0 + (d[k] & 0xffff);
+                const Cx<T> u = d[k] & kGsIn ? w[k] : cx<T>(0, 0);
+#pragma unroll
+                for (int i = 0; i < kGroup; ++i) {
+                    const Cx<T> v = i0 + i < nv ? ld<T>(p, i * x.ss) : cx<T>(0, 0);
+                    acc[2 * i] = fmaT(v.re, u.re, fmaT(v.im, u.im, acc[2 * i]));
+                    acc[2 * i + 1] = fmaT(v.re, u.im, fmaT(-v.im, u.re, acc[2 * i + 1]));
+                }
+            }
+            warp_sums<T, 2 * kGroup>(acc, &sh.red[threadIdx.x >> 5][2 * i0]);
+        }
+        if (pass) norm_share<T, KN>(x, d, w, 2 * nv);
+        cluster_sums<T>(x, 2 * nv + pass, H[pass], pass ? -1 : nv - 2);
+        if (!pass && more) take_rows<T, KN>(x, d, w, nv);
+        v0 = x.V;
+#pragma unroll 1
+        for (int i0 = 0; i0 < nv; i0 += kGroup, v0 += kGroup * x.ss) {
+            Cx<T> c[kGroup];
+#pragma unroll
+            for (int i = 0; i < kGroup; ++i) {
+                c[i] = i0 + i < nv ? cx<T>(-H[pass][2 * (i0 + i)], -H[pass][2 * (i0 + i) + 1]) : cx<T>(0, 0);
+                if (pass) sq += c[i].re * c[i].re + c[i].im * c[i].im;
+            }
+#pragma unroll
+            for (int k = 0; k < KN; ++k) {
+                const vec2<T>* p = v0 + (d[k] & 0xffff);
+#pragma unroll
+                for (int i = 0; i < kGroup; ++i)
+                    w[k] = fma_c(c[i], i0 + i < nv ? ld<T>(p, i * x.ss) : cx<T>(0, 0), w[k]);
+            }
+        }
+    }
+    const T before = H[1][2 * nv];
+    if (sq <= before * T(1.0 / 64)) return before - sq;
+    norm_share<T, KN>(x, d, w, 0);
+    cluster_sums<T>(x, 1, &sh.tmp);
+    return sh.tmp;
+}
+
+// grid (nb * cs), clusters of cs CTAs: problem blockIdx.x / cs.  x (in/out; xzero: from 0) and b at
+// problem offsets pb * N.  KN: nodes a thread at most (own and halo rows).
+template <typename T, int KN>
+__global__ void __launch_bounds__(GsCfg<T>::kThreads) k_gs_step(const __grid_constant__ MArgs<T> a,
+                                                                const vec2<T>* __restrict__ bvec, vec2<T>* xvec,
+                                                                int xzero, int its, int cs) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int NT = blockDim.x;
+    const int pb = blockIdx.x / cs;
+    extern __shared__ __align__(128) unsigned char gs_smem[];
+    GsShared<T>& sh = *reinterpret_cast<GsShared<T>*>(gs_smem);
+    const int n = a.g.n, nn = a.g.nn, tid = threadIdx.x;
+    GsCtx<T> X;
+    X.sh = &sh;
+    X.V = reinterpret_cast<vec2<T>*>(gs_smem + kGsHead<T>);
+    X.rank = blockIdx.x - pb * cs;
+    X.cs = cs;
+    X.W = nn + 2;
+    X.ss = ((nn + cs - 1) / cs + 2) * X.W;
+    X.phase = 0;
+    const int f0 = X.rank * nn / cs;
+    X.R = (X.rank + 1) * nn / cs - f0;
+    const int W = X.W, M = X.R * nn;
+    const vec2<T>* bb = bvec + (long long)pb * a.g.N + (long long)f0 * nn;
+    vec2<T>* xb = xvec + (long long)pb * a.g.N + (long long)f0 * nn;
+    const bool has_up = X.rank > 0, has_dn = X.rank + 1 < cs;
+    const int up = has_up ? nn : 0, dn = has_dn ? nn : 0;
+    unsigned d[KN];
+    Cx<T> w[KN];  // (b at first)
+    auto dirichlet = [&](int i, int j) {
         return (i == 0 && a.g.dir[0]) || (i == n && a.g.dir[1]) || (j == 0 && a.g.dir[2]) || (j == n && a.g.dir[3]);
     };
-    auto val = [&](const vec2<T>* v, int i, int j) {
-        return (i < 0 || i > n || j < 0 || j > n || dirn(i, j)) ? cx<T>(0, 0) : ld<T>(v, (long long)j * nn + i);
-    };
-    // omega D^{-1} (alpha (A v) + beta z) at node (i, j); v == nullptr: v = 0
-    auto dapply = [&](const vec2<T>* v, const vec2<T>* z, Cx<T> alpha, Cx<T> beta, int i, int j) {
-        if (dirn(i, j)) return cx<T>(0, 0);
-        Cx<T> ax = cx<T>(0, 0), dinv_w;
-        const bool fast = i >= 1 && i <= n - 1 && j >= 1 && j <= n - 1;
-        const int tx = i == 0 ? 0 : (i == n ? 2 : 1), ty = j == 0 ? 0 : (j == n ? 2 : 1);
-        if (v) {
-            stencil_node2<T>(c, val(v, i, j - 1), val(v, i, j), val(v, i, j + 1), val(v, i - 1, j - 1),
-                             val(v, i - 1, j), val(v, i - 1, j + 1), val(v, i + 1, j - 1), val(v, i + 1, j),
-                             val(v, i + 1, j + 1), fast, tx, ty, ax, dinv_w);
+    // what depends on nothing before this launch: node words, zeros beside the rows and in the rows
+    // beyond the grid
+    auto coords = [&](int q, int* i, int* j) {
+        if (q < M) {
+            const int r = q / nn;
+            *i = q - r * nn;
+            *j = f0 + r;
         } else {
-            dinv_w = fast ? c.wdinv : c.bdinv[bclass2(tx, ty)];
+            const bool above = q - M < up;
+            *i = q - M - (above ? 0 : up);
+            *j = above ? f0 - 1 : f0 + X.R;
         }
-        const Cx<T> zv = z ? ld<T>(z, (long long)j * nn + i) : cx<T>(0, 0);
-        return cmul(dinv_w, fma_c(alpha, ax, cmul(beta, zv)));
     };
-    const Cx<T> one = cx<T>(1, 0), mone = cx<T>(-1, 0), zero = cx<T>(0, 0);
-    Cx<T> acc[kGsMaxVec];
-    // z0 = omega D^{-1} (b - A x), beta = ||z0||, v_0 = z0 / beta
-    acc[0] = zero;
-    for (long long p = threadIdx.x; p < N; p += kGsCtaThreads) {
-        const int i = (int)(p % nn), j = (int)(p / nn);
-        const Cx<T> w = dapply(xzero ? nullptr : xb, bb, mone, one, i, j);
-        st<T>(W, p, w);
-        acc[0].re += w.re * w.re + w.im * w.im;
-    }
-    cta_sums<T>(acc, 1, red, hc);
-    if (threadIdx.x == 0) {
-        const T beta = sqrt(hc[0].re);
-        scal = beta > T(0) ? T(1) / beta : T(0);
-        g[0] = cx<T>(beta, 0);
-        for (int i = 1; i < kGsMaxVec; ++i) g[i] = zero;
-    }
-    __syncthreads();
-    for (long long p = threadIdx.x; p < N; p += kGsCtaThreads) {
-        const Cx<T> w = ld<T>(W, p);
-        st<T>(V(0), p, cx<T>(w.re * scal, w.im * scal));
-    }
-    __syncthreads();
-    for (int j = 0; j < its; ++j) {
-        const vec2<T>* vj = V(j);
-        for (long long p = threadIdx.x; p < N; p += kGsCtaThreads) {
-            const int i = (int)(p % nn), jj = (int)(p / nn);
-            st<T>(W, p, dapply(vj, nullptr, one, zero, i, jj));
+#pragma unroll
+    for (int k = 0; k < KN; ++k) {
+        const int q = tid + k * NT;
+        d[k] = 0;
+        if (q < M + up + dn) {
+            int i, j;
+            coords(q, &i, &j);
+            const int r = j - f0;
+            const int tx = i == 0 ? 0 : (i == n ? 2 : 1), ty = j == 0 ? 0 : (j == n ? 2 : 1);
+            d[k] = (unsigned)((r + 1) * W + i + 1);
+            if (q < M)
+                d[k] |= (unsigned)(tx == 1 && ty == 1 ? 8 : bclass2(tx, ty)) << 16 | (has_up && r == 0 ? kGsUp : 0) |
+                        (has_dn && r == X.R - 1 ? kGsDn : 0) | (dirichlet(i, j) ? 0 : kGsFree) | kGsIn;
+            else
+                d[k] |= kGsHalo;
         }
-        __syncthreads();
-        // classical Gram-Schmidt, twice
-        for (int pass = 0; pass < 2; ++pass) {
-            for (int i = 0; i <= j; ++i) acc[i] = zero;
-            for (long long p = threadIdx.x; p < N; p += kGsCtaThreads) {
-                const Cx<T> w = ld<T>(W, p);
-                for (int i = 0; i <= j; ++i) {
-                    const Cx<T> v = ld<T>(V(i), p);
-                    acc[i].re += v.re * w.re + v.im * w.im;
-                    acc[i].im += v.re * w.im - v.im * w.re;
-                }
-            }
-            cta_sums<T>(acc, j + 1, red, hc);
-            if ((int)threadIdx.x <= j) R[threadIdx.x][j] = pass ? R[threadIdx.x][j] + hc[threadIdx.x] : hc[threadIdx.x];
-            acc[0] = zero;
-            for (long long p = threadIdx.x; p < N; p += kGsCtaThreads) {
-                Cx<T> w = ld<T>(W, p);
-                for (int i = 0; i <= j; ++i) w = fma_c(cx<T>(-hc[i].re, -hc[i].im), ld<T>(V(i), p), w);
-                st<T>(W, p, w);
-                acc[0].re += w.re * w.re + w.im * w.im;
-            }
-            __syncthreads();
-        }
-        cta_sums<T>(acc, 1, red, hc);  // ||w||^2 after the second pass
-        if (threadIdx.x == 0) {
-            const T h = sqrt(hc[0].re);
-            scal = h > T(0) ? T(1) / h : T(0);
-            // previous rotations on column j, then the one that zeroes h
-            for (int i = 0; i < j; ++i) {
-                const Cx<T> p0 = R[i][j], q0 = R[i + 1][j];
-                const T cc = csv[i];
-                const Cx<T> s0 = sn[i];
-                R[i][j] = cx<T>(cc * p0.re + (s0.re * q0.re - s0.im * q0.im), cc * p0.im + (s0.re * q0.im + s0.im * q0.re));
-                R[i + 1][j] = cx<T>(-(s0.re * p0.re + s0.im * p0.im) + cc * q0.re, -(s0.re * p0.im - s0.im * p0.re) + cc * q0.im);
-            }
-            const Cx<T> av = R[j][j];
-            const T na = sqrt(av.re * av.re + av.im * av.im), den = sqrt(na * na + h * h);
-            T cc = T(1);
-            Cx<T> s0 = zero;
-            if (den > T(0)) {
-                if (na == T(0)) {
-                    cc = T(0);
-                    s0 = one;
-                } else {
-                    cc = na / den;
-                    s0 = cx<T>(av.re / na * h / den, av.im / na * h / den);
-                }
-            }
-            csv[j] = cc;
-            sn[j] = s0;
-            R[j][j] = cx<T>(cc * av.re + s0.re * h, cc * av.im + s0.im * h);
-            const Cx<T> g0 = g[j];
-            g[j] = cx<T>(cc * g0.re, cc * g0.im);
-            g[j + 1] = cx<T>(-(s0.re * g0.re + s0.im * g0.im), -(s0.re * g0.im - s0.im * g0.re));
-        }
-        __syncthreads();
-        vec2<T>* vn = V(j + 1);
-        for (long long p = threadIdx.x; p < N; p += kGsCtaThreads) {
-            const Cx<T> w = ld<T>(W, p);
-            st<T>(vn, p, cx<T>(w.re * scal, w.im * scal));
-        }
-        __syncthreads();
+        if (KN > 2 && __all_sync(0xffffffffu, (d[k] >> 16 & 15) == 8)) d[k] |= kGsInner;
     }
-    if (threadIdx.x == 0) {
-        for (int j = its - 1; j >= 0; --j) {
-            Cx<T> t = g[j];
-            for (int k = j + 1; k < its; ++k) t = t - cmul(R[j][k], ys[k]);
-            const Cx<T> d = R[j][j];
-            const T dd = d.re * d.re + d.im * d.im;
-            ys[j] = dd > T(0) ? cx<T>((t.re * d.re + t.im * d.im) / dd, (t.im * d.re - t.re * d.im) / dd) : zero;
+    {
+        const int slots = max(its, 2), rows = X.R + 2;
+        for (int t = tid; t < slots * rows; t += NT) {
+            const int q = t / rows, r = t - q * rows;
+            vec2<T>* row = X.V + q * X.ss + r * W;
+            st<T>(row, 0, cx<T>(0, 0));
+            st<T>(row, W - 1, cx<T>(0, 0));
+        }
+        for (int t = tid; t < W; t += NT)
+            for (int q = 0; q < slots; ++q) {
+                if (!has_up) st<T>(X.V, q * X.ss + t, cx<T>(0, 0));
+                if (!has_dn) st<T>(X.V, q * X.ss + (X.R + 1) * W + t, cx<T>(0, 0));
+            }
+    }
+    if (cs > 1) {
+        cg::this_cluster().sync();  // every CTA is in place
+        const int ru = has_up ? f0 - (X.rank - 1) * nn / cs : 0;  // rows of the CTA above
+        X.vup = has_up ? cg::this_cluster().map_shared_rank(X.V, X.rank - 1) + ru * W : nullptr;
+        X.vdn = has_dn ? cg::this_cluster().map_shared_rank(X.V, X.rank + 1) - X.R * W : nullptr;
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (a.pc && problem_skipped(a, pb)) return;  // the whole cluster
+    if (tid < 9) {
+        const PCoef<T>& c = a.pc ? a.pc[pb] : a.c0;
+        GsWeights<T>& k = sh.wt[tid];
+        const bool in = tid == 8;
+        k.w[0] = in ? c.iw[0] : c.bw[tid][0];
+        k.w[1] = in ? c.iw[1] : c.bw[tid][1];
+        k.w[2] = in ? c.iw[1] : c.bw[tid][2];
+        k.w[3] = in ? c.iw[2] : c.bw[tid][3];
+        k.dinv = in ? c.wdinv : c.bdinv[tid];
+    }
+    // b; x with its halo rows to basis vector 1 (first written when every CTA is past its use here)
+#pragma unroll
+    for (int k = 0; k < KN; ++k) {
+        w[k] = d[k] & kGsFree ? ld<T>(bb, tid + k * NT) : cx<T>(0, 0);
+        if (!xzero && d[k]) {
+            int i, j;
+            coords(tid + k * NT, &i, &j);
+            st<T>(X.V, X.ss + (d[k] & 0xffff),
+                  dirichlet(i, j) ? cx<T>(0, 0) : ld<T>(xb, (long long)(j - f0) * nn + i));
         }
     }
     __syncthreads();
-    for (long long p = threadIdx.x; p < N; p += kGsCtaThreads) {
-        Cx<T> u = xzero ? zero : ld<T>(xb, p);
-        for (int i = 0; i < its; ++i) u = fma_c(ys[i], ld<T>(V(i), p), u);
-        st<T>(xb, p, u);
+    // z0 = omega D^{-1} (b - A x), beta = ||z0||, v_0 = z0 / beta; then w = omega D^{-1} A v_j
+#pragma unroll 1
+    for (int j = -1; j < its; ++j) {
+        const bool more = j + 1 < its;
+        T h2;
+        // (keeps every node's addresses from being worked out before the loop, and spilled)
+#pragma unroll
+        for (int k = 0; k < KN; ++k) asm volatile("" : "+r"(d[k]));
+        if (j >= 0 || !xzero) {
+            const vec2<T>* f = X.V + (j < 0 ? 1 : j) * X.ss;
+#pragma unroll
+            for (int k = 0; k < KN; ++k) {
+                // (a node without an unknown applies the stencil at a place where it can)
+                Cx<T> dinv;
+                const bool fr = d[k] & kGsFree;
+                const Cx<T> ax = band_apply<T>(sh.wt, f, W, fr ? d[k] : (unsigned)(W + 1) | 8u << 16, &dinv);
+                const Cx<T> v = cmul(dinv, j < 0 ? w[k] - ax : ax);
+                w[k] = fr ? v : cx<T>(0, 0);
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < KN; ++k)
+                if (d[k] & kGsFree) w[k] = cmul(sh.wt[(d[k] >> 16) & 15].dinv, w[k]);
+        }
+        if (j >= 0) {
+            h2 = orthogonalise<T, KN>(X, d, w, j + 1, more);
+        } else {
+            send_rows<T, KN>(X, d, w, 0);
+            norm_share<T, KN>(X, d, w, 0);
+            cluster_sums<T>(X, 1, &sh.beta2);
+            take_rows<T, KN>(X, d, w, 0);
+            h2 = sh.beta2;
+        }
+        const T h = sqrt(h2);
+        if (tid == 0) {
+            if (j >= 0)
+                sh.h[j] = h;
+            else
+                sh.g[0] = cx<T>(h, 0);
+        }
+        if (!more) break;
+        const T s = h > T(0) ? T(1) / h : T(0);
+        vec2<T>* vn = X.V + (j + 1) * X.ss;
+#pragma unroll
+        for (int k = 0; k < KN; ++k)
+            if (d[k]) st<T>(vn, d[k] & 0xffff, cx<T>(w[k].re * s, w[k].im * s));
+        __syncthreads();
     }
+    // x early: its latency runs beside the small problem
+#pragma unroll
+    for (int k = 0; k < KN; ++k) w[k] = !xzero && (d[k] & kGsIn) ? ld<T>(xb, tid + k * NT) : cx<T>(0, 0);
+    if (tid < 32) {
+        if (tid == 0) rotate_column<T>(sh, its - 1);
+        __syncwarp();
+        back_substitute<T>(sh, its);
+    }
+    __syncthreads();
+    for (int i = 0; i < its; ++i) {
+        const Cx<T> y = sh.ys[i];
+#pragma unroll
+        for (int k = 0; k < KN; ++k) w[k] = fma_c(y, ld<T>(X.V, i * X.ss + (d[k] & 0xffff)), w[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < KN; ++k)
+        if (d[k] & kGsIn) st<T>(xb, tid + k * NT, w[k]);
+}
+
+template <typename T, int KN>
+int gs_cluster_of() {
+    if (cudaFuncSetAttribute(k_gs_step<T, KN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGsSmemMax) !=
+        cudaSuccess)
+        return -1;
+    cudaFuncSetAttribute(k_gs_step<T, KN>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    for (int cs = kGsClusterMax; cs > 1; cs >>= 1) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)cs);
+        cfg.blockDim = dim3(GsCfg<T>::kThreads);
+        cfg.dynamicSmemBytes = kGsSmemMax;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)cs;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int active = 0;
+        if (cudaOccupancyMaxActiveClusters(&active, k_gs_step<T, KN>, &cfg) == cudaSuccess && active >= 1) return cs;
+    }
+    return 1;
+}
+
+// Configure k_gs_step<T> and find the largest cluster of it that the device holds (once per device).
+template <typename T>
+int gs_cluster_max() {
+    constexpr int kMaxDev = 64;
+    static std::mutex mu;
+    static int held[kMaxDev];  // 0: not looked at yet, -1: not available
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) {
+        cudaGetLastError();
+        return -1;
+    }
+    std::lock_guard<std::mutex> g(mu);
+    if (!held[dev]) {
+        held[dev] = std::min({gs_cluster_of<T, 1>(), gs_cluster_of<T, 2>(), gs_cluster_of<T, 5>()});
+        cudaGetLastError();
+    }
+    return held[dev];
+}
+
+// nodes of the largest band with its halo rows
+inline long long gs_band(int nn, int cs) { return (long long)((nn + cs - 1) / cs + (cs > 1 ? 2 : 0)) * nn; }
+
+template <typename T>
+size_t gs_step_smem(int nn, int its, int cs) {
+    const size_t rows = (size_t)(nn + cs - 1) / cs;
+    return kGsHead<T> + (size_t)std::max(its, 2) * (rows + 2) * (nn + 2) * sizeof(vec2<T>);
 }
 
 }  // namespace
 
 template <typename T>
-cudaError_t launch_gs_cta(const MArgs<T>& a, const vec2<T>* b, vec2<T>* x, int xzero, int its, vec2<T>* V,
-                          long long ldv, cudaStream_t s) {
-    if (a.g.dim != 2 || its < 1 || its > kGsMaxIts || a.g.N > kGsCtaNodes) return cudaErrorInvalidValue;
-    if (!a.pc && a.nb != 1) return cudaErrorInvalidValue;
-    return klaunch(k_gs_cta<T>, dim3((unsigned)a.nb), dim3(kGsCtaThreads), 0, s, 1, a, b, x, xzero, its, V, ldv);
+int gs_step_cluster(const GridDesc& g, int its) {
+    if (g.dim != 2 || its < 1 || its > kGsMaxIts) return 0;
+    const int most = gs_cluster_max<T>();
+    int best = 0;
+    for (int cs = 1; cs <= most && cs <= g.nn; cs <<= 1) {
+        const long long nodes = gs_band(g.nn, cs);
+        if (nodes > 5LL * GsCfg<T>::kThreads || gs_step_smem<T>(g.nn, its, cs) > kGsSmemMax) continue;
+        best = cs;
+        if (nodes <= kGsBand) break;
+    }
+    return best;
+}
+
+template <typename T>
+cudaError_t launch_gs_step(const MArgs<T>& a, const vec2<T>* b, vec2<T>* x, int xzero, int its, int cs,
+                           cudaStream_t s) {
+    if (cs < 1 || (!a.pc && a.nb != 1)) return cudaErrorInvalidValue;
+    const long long nodes = gs_band(a.g.nn, cs);
+    // complex64: a warp per scalar of a sum at least, for the sums over the warps are a serial chain
+    // (751 -> 712 us with the set-up before the wait for the previous kernel); complex128: as few as the
+    // nodes need, for each costs the FP64 pipe its time
+    const int most = GsCfg<T>::kThreads;
+    const int least = sizeof(T) == 8 ? 64 : std::min(most, 32 * (2 * its + 1));
+    const int kn = nodes <= most ? 1 : nodes <= 2 * most ? 2 : 5;
+    const dim3 grd((unsigned)(a.nb * cs));
+    const dim3 blk((unsigned)std::max((long long)least, ((nodes + kn - 1) / kn + 31) / 32 * 32));
+    const size_t sm = gs_step_smem<T>(a.g.nn, its, cs);
+    if (kn == 1) return klaunch(k_gs_step<T, 1>, grd, blk, sm, s, cs, a, b, x, xzero, its, cs);
+    if (kn == 2) return klaunch(k_gs_step<T, 2>, grd, blk, sm, s, cs, a, b, x, xzero, its, cs);
+    return klaunch(k_gs_step<T, 5>, grd, blk, sm, s, cs, a, b, x, xzero, its, cs);
 }
 
 template <typename T>
@@ -502,10 +877,12 @@ cudaError_t launch_gs_update(vec2<T>* x, const vec2<T>* V, long long ld, int m, 
                                             const Batch&, cudaStream_t);                                              \
     template cudaError_t launch_gs_update<T>(vec2<T>*, const vec2<T>*, long long, int, long long, const double2*,     \
                                              int, const Batch&, cudaStream_t);
-template cudaError_t launch_gs_cta<float>(const MArgs<float>&, const vec2<float>*, vec2<float>*, int, int,
-                                          vec2<float>*, long long, cudaStream_t);
-template cudaError_t launch_gs_cta<double>(const MArgs<double>&, const vec2<double>*, vec2<double>*, int, int,
-                                           vec2<double>*, long long, cudaStream_t);
+template int gs_step_cluster<float>(const GridDesc&, int);
+template int gs_step_cluster<double>(const GridDesc&, int);
+template cudaError_t launch_gs_step<float>(const MArgs<float>&, const vec2<float>*, vec2<float>*, int, int, int,
+                                           cudaStream_t);
+template cudaError_t launch_gs_step<double>(const MArgs<double>&, const vec2<double>*, vec2<double>*, int, int, int,
+                                            cudaStream_t);
 HH_GS_INST(float)
 HH_GS_INST(double)
 #undef HH_GS_INST
