@@ -327,9 +327,14 @@ static int band_rows(const GridDesc& g, int nsweeps, int want) {
 }
 
 static int g_cluster_size = 0;
+static int g_fit_size3 = 0;  // cluster size that decides which 3D levels run in a cluster (coarse_fits)
 
 int coarse_cluster_size() {
     if (g_cluster_size) return g_cluster_size;
+    cudaFuncAttributes fa = {};
+    const bool single_only = cudaFuncGetAttributes(&fa, k_coarse_dsmem<float>) != cudaSuccess ||
+                             fa.maxDynamicSharedSizeBytes < (int)kCoarseSmemMax;
+    cudaGetLastError();
     // the query below asks for kCoarseSmemMax, which the queried kernel has to be allowed: where only the
     // complex128 kernels had been prepared it failed and the level ran in one CTA (33^2: 128 us)
     cudaFuncSetAttribute(k_coarse_dsmem<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmemMax);
@@ -352,11 +357,13 @@ int coarse_cluster_size() {
     cfg.numAttrs = 1;
     int nclusters = 0;
     if (cudaOccupancyMaxActiveClusters(&nclusters, k_coarse_dsmem<float>, &cfg) == cudaSuccess && nclusters >= 1) {
+        g_fit_size3 = single_only ? 1 : cs;
         g_cluster_size = cs;
         return cs;
     }
     cudaGetLastError();
     }
+    g_fit_size3 = 1;
     g_cluster_size = 1;
     return 1;
 }
@@ -370,9 +377,14 @@ bool coarse_cluster_ok(const GridDesc& g, int cs) {
     return sp.smem <= kCoarseSmemMax && rows * sp.S <= cta_capacity(g);
 }
 
+// In 2D the cluster's sweeps equal the separate ones bit for bit.  The 3D ones add the neighbours in
+// another order than the tile kernels, so a level that moved from one to the other would change in its
+// last digits: in a process whose first problem is complex128, where no cluster was found before the
+// query above was right, the 3D levels beyond one CTA stay with separate sweeps.
 template <typename T>
 bool coarse_fits(const GridDesc& g) {
-    return coarse_cluster_ok<T>(g, coarse_cluster_size());
+    const int cs = coarse_cluster_size();
+    return coarse_cluster_ok<T>(g, g.dim == 3 ? g_fit_size3 : cs);
 }
 
 template <typename T>
