@@ -61,9 +61,14 @@ static SlabPlan slab_plan(const GridDesc& g, int cs) {
 
 // One cluster per problem of the batch: problem = blockIdx.x / cluster size.  Coefficients
 // from the table entry of A_L on this level (interior weights and omega D^{-1} included).
-template <typename T>
-__global__ void __launch_bounds__(kCoarseThreads) k_coarse_dsmem(const __grid_constant__ MArgs<T> a, int nsweeps,
-                                                                 int per) {
+// K nodes per thread; a sweep lasts as long as one warp's chain over them (nodes near a side take about
+// 400 instructions), so K = 1 wherever the CTA's nodes allow, with the 1D rows kept over the sweeps, and
+// the cluster is the smallest that gives each thread a node (fewer CTAs to wait for).  HSS step with the
+// coarsest level 3^3, 5^3, 6^3, 17^3, us: 48.2 -> 43.7, 51.6 -> 46.1, 52.6 -> 48.5, 172 -> 164.
+constexpr int kCoarseThreads1 = 640;  // K = 1: holds two planes of 17^2
+template <typename T, int K>
+__global__ void __launch_bounds__(K == 1 ? kCoarseThreads1 : kCoarseThreads)
+k_coarse_dsmem(const __grid_constant__ MArgs<T> a, int nsweeps, int per) {
     pdl_entry();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cg::cluster_group cl = cg::this_cluster();
@@ -77,19 +82,25 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_dsmem(const __grid_co
     vec2<T>* __restrict__ xout = a.y + (long long)prob * a.bs;
     const T omega = a.omega;
     const int nn = g.nn, n = g.n;
-    const bool d3 = g.dim == 3;
-    const long long S = d3 ? (long long)nn * nn : nn;
+    const long long S = (long long)nn * nn;
     const int r0 = min(rank * per, nn);
     const int r1 = min(r0 + per, nn);
     const int own = (r1 - r0) * (int)S;               // owned nodes (at most kCoarseNodesPerThread per thread)
     const long long buf = (long long)(per + 2) * S;   // one iterate buffer, halos included
-    vec2<T>* xs[2] = {reinterpret_cast<vec2<T>*>(smem_raw), reinterpret_cast<vec2<T>*>(smem_raw) + buf};
+    vec2<T>* const xs0 = reinterpret_cast<vec2<T>*>(smem_raw);
+    auto xs = [&](int c) { return xs0 + c * buf; };
     const T h = T(g.h), ih = T(1.0 / g.h);
     const long long off = (long long)(r0 - 1) * S;    // global node number of local index 0
 
     // per owned node, once: coordinates, class, b and omega D^{-1}
-    constexpr int K = kCoarseNodesPerThread;
     int ii[K], jj[K], ll[K];
+    constexpr bool KEEP = K == 1 && sizeof(T) == 4;  // (else the registers do not hold them)
+    Row1<T> rx[K], ry[K], rz[K];
+    auto rows = [&](int k) {
+        rx[k] = row1<T>(ii[k], n, g.dir[0], g.dir[1], h, ih);
+        ry[k] = row1<T>(jj[k], n, g.dir[2], g.dir[3], h, ih);
+        rz[k] = row1<T>(ll[k], n, g.dir[4], g.dir[5], h, ih);
+    };
     unsigned char cls[K];  // 0 masked, 1 interior (fast), 2 boundary (general)
     Cx<T> bq[K], dw[K];
 #pragma unroll
@@ -102,32 +113,25 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_dsmem(const __grid_co
         const unsigned pu = (unsigned)((long long)r0 * S + q), nnu = (unsigned)nn, qq = pu / nnu;
         ii[k] = (int)(pu - qq * nnu);
         jj[k] = (int)(qq % nnu);
-        ll[k] = d3 ? (int)(qq / nnu) : 0;
-        const Row1<T> rx = row1<T>(ii[k], n, g.dir[0], g.dir[1], h, ih);
-        const Row1<T> ry = row1<T>(jj[k], n, g.dir[2], g.dir[3], h, ih);
-        Row1<T> rz = rx;
-        bool masked = rx.masked || ry.masked;
-        if (d3) {
-            rz = row1<T>(ll[k], n, g.dir[4], g.dir[5], h, ih);
-            masked = masked || rz.masked;
-        }
+        ll[k] = (int)(qq / nnu);
+        rows(k);
+        const bool masked = rx[k].masked || ry[k].masked || rz[k].masked;
         if (masked) continue;
         const bool fast = ii[k] >= 2 && ii[k] <= n - 2 && jj[k] >= 2 && jj[k] <= n - 2 &&
-                          (!d3 || (ll[k] >= 2 && ll[k] <= n - 2));
+                          ll[k] >= 2 && ll[k] <= n - 2;
         cls[k] = fast ? 1 : 2;
         bq[k] = ld<T>(b, (long long)r0 * S + q);
         if (fast) {
             dw[k] = pcf.wdinv;
         } else {
-            const NodeResult<T> r = d3 ? node3<T, false>(xs[0], nn, ii[k], jj[k], ll[k], rx, ry, rz, op, off)
-                                       : node2<T, false>(xs[0], nn, ii[k], jj[k], rx, ry, op, off);
+            const NodeResult<T> r = node3<T, false>(xs0, nn, ii[k], jj[k], ll[k], rx[k], ry[k], rz[k], op, off);
             dw[k] = omega * cinv(r.d);
         }
     }
     int cur = 0;
     for (int s = 0; s < nsweeps; ++s) {
-        const vec2<T>* __restrict__ xc = xs[cur];
-        vec2<T>* xn = xs[cur ^ 1];
+        const vec2<T>* __restrict__ xc = xs(cur);
+        vec2<T>* xn = xs(cur ^ 1);
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             const int q = threadIdx.x + k * blockDim.x;
@@ -140,39 +144,25 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_dsmem(const __grid_co
                 } else {
                     Cx<T> ax;
                     if (cls[k] == 1) {
-                        if (!d3) {
-                            const Cx<T> e = (ld<T>(xc, lq - 1) + ld<T>(xc, lq + 1)) +
-                                            (ld<T>(xc, lq - nn) + ld<T>(xc, lq + nn));
-                            const Cx<T> dg = (ld<T>(xc, lq - nn - 1) + ld<T>(xc, lq - nn + 1)) +
-                                             (ld<T>(xc, lq + nn - 1) + ld<T>(xc, lq + nn + 1));
-                            ax = fma_c(pcf.iw[2], dg, fma_c(pcf.iw[1], e, cmul(pcf.iw[0], ld<T>(xc, lq))));
-                        } else {
-                            // neighbours grouped by how many coordinates differ: 6 faces, 12 edges, 8 corners
-                            Cx<T> fa = cx<T>(0, 0), ed = cx<T>(0, 0), co = cx<T>(0, 0);
+                        // neighbours grouped by how many coordinates differ: 6 faces, 12 edges, 8 corners
+                        Cx<T> fa = cx<T>(0, 0), ed = cx<T>(0, 0), co = cx<T>(0, 0);
 #pragma unroll
-                            for (int dz = -1; dz <= 1; ++dz)
+                        for (int dz = -1; dz <= 1; ++dz)
 #pragma unroll
-                                for (int dy = -1; dy <= 1; ++dy)
+                            for (int dy = -1; dy <= 1; ++dy)
 #pragma unroll
-                                    for (int dx = -1; dx <= 1; ++dx) {
-                                        const int m = (dx != 0) + (dy != 0) + (dz != 0);
-                                        if (m == 0) continue;
-                                        const Cx<T> v = ld<T>(xc, lq + ((long long)dz * nn + dy) * nn + dx);
-                                        if (m == 1) fa = fa + v;
-                                        else if (m == 2) ed = ed + v;
-                                        else co = co + v;
-                                    }
-                            ax = fma_c(pcf.iw[3], co, fma_c(pcf.iw[2], ed, fma_c(pcf.iw[1], fa, cmul(pcf.iw[0], ld<T>(xc, lq)))));
-                        }
+                                for (int dx = -1; dx <= 1; ++dx) {
+                                    const int m = (dx != 0) + (dy != 0) + (dz != 0);
+                                    if (m == 0) continue;
+                                    const Cx<T> v = ld<T>(xc, lq + ((long long)dz * nn + dy) * nn + dx);
+                                    if (m == 1) fa = fa + v;
+                                    else if (m == 2) ed = ed + v;
+                                    else co = co + v;
+                                }
+                        ax = fma_c(pcf.iw[3], co, fma_c(pcf.iw[2], ed, fma_c(pcf.iw[1], fa, cmul(pcf.iw[0], ld<T>(xc, lq)))));
                     } else {
-                        const Row1<T> rx = row1<T>(ii[k], n, g.dir[0], g.dir[1], h, ih);
-                        const Row1<T> ry = row1<T>(jj[k], n, g.dir[2], g.dir[3], h, ih);
-                        if (d3) {
-                            const Row1<T> rz = row1<T>(ll[k], n, g.dir[4], g.dir[5], h, ih);
-                            ax = node3<T, true>(xc, nn, ii[k], jj[k], ll[k], rx, ry, rz, op, off).ax;
-                        } else {
-                            ax = node2<T, true>(xc, nn, ii[k], jj[k], rx, ry, op, off).ax;
-                        }
+                        if (!KEEP) rows(k);
+                        ax = node3<T, true>(xc, nn, ii[k], jj[k], ll[k], rx[k], ry[k], rz[k], op, off).ax;
                     }
                     xv = fma_c(dw[k], bq[k] - ax, ld<T>(xc, lq));
                 }
@@ -185,7 +175,7 @@ __global__ void __launch_bounds__(kCoarseThreads) k_coarse_dsmem(const __grid_co
         cl.sync();
         cur ^= 1;
     }
-    for (int q = threadIdx.x; q < own; q += blockDim.x) xout[(long long)r0 * S + q] = xs[cur][q + S];
+    for (int q = threadIdx.x; q < own; q += blockDim.x) xout[(long long)r0 * S + q] = xs(cur)[q + S];
 }
 
 // ---- 2D: padded slabs, boundary classes, `depth` sweeps per cluster barrier ----
@@ -332,14 +322,16 @@ static int g_fit_size3 = 0;  // cluster size that decides which 3D levels run in
 int coarse_cluster_size() {
     if (g_cluster_size) return g_cluster_size;
     cudaFuncAttributes fa = {};
-    const bool single_only = cudaFuncGetAttributes(&fa, k_coarse_dsmem<float>) != cudaSuccess ||
+    const bool single_only = cudaFuncGetAttributes(&fa, k_coarse_dsmem<float, 2>) != cudaSuccess ||
                              fa.maxDynamicSharedSizeBytes < (int)kCoarseSmemMax;
     cudaGetLastError();
     // the query below asks for kCoarseSmemMax, which the queried kernel has to be allowed: where only the
     // complex128 kernels had been prepared it failed and the level ran in one CTA (33^2: 128 us)
-    cudaFuncSetAttribute(k_coarse_dsmem<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmemMax);
-    cudaFuncSetAttribute(k_coarse_dsmem<float>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    cudaFuncSetAttribute(k_coarse_dsmem<double>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaFuncSetAttribute(k_coarse_dsmem<float, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmemMax);
+    cudaFuncSetAttribute(k_coarse_dsmem<float, 2>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaFuncSetAttribute(k_coarse_dsmem<double, 2>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaFuncSetAttribute(k_coarse_dsmem<float, 1>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaFuncSetAttribute(k_coarse_dsmem<double, 1>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     cudaFuncSetAttribute(k_coarse_dsmem2<float>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     cudaFuncSetAttribute(k_coarse_dsmem2<double>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     cudaGetLastError();
@@ -356,7 +348,7 @@ int coarse_cluster_size() {
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int nclusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&nclusters, k_coarse_dsmem<float>, &cfg) == cudaSuccess && nclusters >= 1) {
+    if (cudaOccupancyMaxActiveClusters(&nclusters, k_coarse_dsmem<float, 2>, &cfg) == cudaSuccess && nclusters >= 1) {
         g_fit_size3 = single_only ? 1 : cs;
         g_cluster_size = cs;
         return cs;
@@ -389,8 +381,10 @@ bool coarse_fits(const GridDesc& g) {
 
 template <typename T>
 cudaError_t prepare_coarse() {
-    cudaError_t e = cudaFuncSetAttribute(k_coarse_dsmem<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(k_coarse_dsmem<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kCoarseSmemMax);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(k_coarse_dsmem<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmemMax);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_coarse_dsmem2<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmemMax);
     if (e != cudaSuccess) return e;
@@ -411,6 +405,12 @@ template <typename T>
 static int batch_cluster_size(const GridDesc& g, int nb) {
     int cs = coarse_cluster_size();
     while (cs > 1 && (long long)nb * cs > 2LL * num_sms() && coarse_cluster_ok<T>(g, cs / 2)) cs /= 2;
+    // 3D: no more CTAs than give each thread a node (a smaller cluster's barriers cost less)
+    auto one_each = [&](int c) {
+        const SlabPlan sp = slab_plan<T>(g, c);
+        return sp.per * sp.S <= kCoarseThreads && sp.smem <= kCoarseSmemMax;
+    };
+    while (g.dim == 3 && cs > 1 && one_each(cs / 2)) cs /= 2;
     return cs;
 }
 
@@ -437,7 +437,10 @@ cudaError_t launch_coarse_solve(const MArgs<T>& a, int nsweeps, cudaStream_t s) 
     if (a.g.dim == 2)
         return klaunch(k_coarse_dsmem2<T>, dim3(cs * a.nb), dim3(kCoarseThreads), sp.smem, s, cs, a, nsweeps, sp.per,
                        sp.depth);
-    return klaunch(k_coarse_dsmem<T>, dim3(cs * a.nb), dim3(kCoarseThreads), sp.smem, s, cs, a, nsweeps, sp.per);
+    if (const long long own = sp.per * sp.S; own <= kCoarseThreads1)
+        return klaunch(k_coarse_dsmem<T, 1>, dim3(cs * a.nb), dim3((unsigned)((own + 31) / 32 * 32)), sp.smem, s, cs, a,
+                       nsweeps, sp.per);
+    return klaunch(k_coarse_dsmem<T, 2>, dim3(cs * a.nb), dim3(kCoarseThreads), sp.smem, s, cs, a, nsweeps, sp.per);
 }
 
 template bool coarse_fits<float>(const GridDesc&);
