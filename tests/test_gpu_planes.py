@@ -27,7 +27,7 @@ def test_planes_and_fused_prolongation(libhh, n, levels, nu_post, bc, nb):
         o = hh.default_options(levels=levels, nu_post=nu_post, restart=2, tile_rows=rows)
         g = torch.Generator(device="cuda").manual_seed(n)
         with hh.Problem(3, n, k, 0.0, k, bc, o) as p:
-            r = torch.randn(p.size() * nb, dtype=torch.complex128, device="cuda", generator=g)
+            r = torch.randn(p.size(), dtype=torch.complex128, device="cuda", generator=g)
             out.append([p.precondition(r), p.precondition(r), p.vcycle(r.to(torch.complex64))])
     for a, b in zip(*out):
         assert torch.equal(a, b)
