@@ -217,6 +217,8 @@ cudaError_t launch_march2rr(int mode, const MArgs<T>& a, cudaStream_t s);
 
 // ---- 3D tile kernels (march3.cu): modes M_APPLY, M_AXPBY, M_DAXPBY, M_JACOBI, M_HSS_FIRST and
 //      M_JACOBI2_ZERO ----
+// planes per tile of the complex64 kernels for nb problems on grid g, unless a.tile_rows says
+int march3_planes(const GridDesc& g, int nb);
 template <typename T>
 cudaError_t launch_march3(int mode, const MArgs<T>& a, cudaStream_t s);
 

@@ -299,21 +299,23 @@ static cudaError_t go3(MArgs<T> a, cudaStream_t s) {
     return klaunch(k_march3<T, MODE, R, false>, grd, dim3(32 * kWarps3), smem, s, 1, a, zt);
 }
 
+// Planes per tile of the complex64 kernels (the results do not depend on them).  4 where the grid fills
+// the chip (257^3: 8 halve the resident CTAs, 2 double the halo planes); a grid of few tiles is bound by
+// the chain of one tile, which shortens with its planes.  HSS step of the 3D preconditioner with 4, 2, 1
+// planes on every level, us: 41^3 72, 58, 53; 49^3 74, 61, 62 (234 tiles of 4); 65^3 79, 74, 77 (561);
+// 97^3 108, 110 (1700); 129^3 168, 200.
+int march3_planes(const GridDesc& g, int nb) {
+    const long long nn = g.nn, sms = num_sms();
+    const long long tiles = ((nn + 29) / 30) * ((nn + kWarps3 - 3) / (kWarps3 - 2)) * ((nn + 3) / 4) * nb;
+    return 3 * tiles <= 4 * sms ? 1 : (tiles <= 2 * sms ? 2 : 4);
+}
+
 template <typename T, int MODE>
 static cudaError_t pick3(MArgs<T> a, cudaStream_t s) {
     a.h = T(a.g.h);
     a.ih = T(1.0 / a.g.h);
     if constexpr (sizeof(T) == 4) {
-        // Planes per tile (the results do not depend on them).  4 where the grid fills the chip (257^3: 8
-        // halve the resident CTAs, 2 double the halo planes); a grid of few tiles is bound by the chain of
-        // one tile, which shortens with its planes.  HSS step of the 3D preconditioner with 4, 2, 1 planes
-        // on every level, us: 41^3 72, 58, 53; 49^3 74, 61, 62 (234 tiles of 4); 65^3 79, 74, 77 (561);
-        // 97^3 108, 110 (1700); 129^3 168, 200.
-        const long long nn = a.g.nn, sms = num_sms();
-        const long long tiles = ((nn + 29) / 30) * ((nn + kWarps3 - 3) / (kWarps3 - 2)) * ((nn + 3) / 4) * a.nb;
-        int R = a.tile_rows;
-        if (R == 0) R = 3 * tiles <= 4 * sms ? 1 : (tiles <= 2 * sms ? 2 : 4);
-        switch (R) {
+        switch (a.tile_rows ? a.tile_rows : march3_planes(a.g, a.nb)) {
             case 1: return go3<T, MODE, 1>(a, s);
             case 2: return go3<T, MODE, 2>(a, s);
             case 8: return go3<T, MODE, 8>(a, s);
