@@ -79,14 +79,16 @@ __global__ void __launch_bounds__(256) k_restrict(GridDesc gc, const vec2<T>* __
 
 // 3D: every load of a node is in flight before the first addition; plane by plane the pass cost three
 // trips to L2 (11^3 .. 33^3 coarse nodes 5.5 .. 6.6 us, now about 3).  With the same change in
-// k_prolong3 an HSS step on 41^3 went from 83 to 73 us, on 129^3 from 185 to 174.
+// k_prolong3 an HSS step on 41^3 went from 83 to 73 us, on 129^3 from 185 to 174.  Nodes are numbered
+// through the plane: rows of 2^m + 1 nodes do not fill warps (residual and restriction on 257^3
+// 159 -> 155 us, 129^3 28.8 -> 26.9).
 template <typename T>
 __global__ void __launch_bounds__(256) k_restrict3(GridDesc gc, const vec2<T>* __restrict__ rf, vec2<T>* __restrict__ rc,
                                                    Batch bt) {
     pdl_entry();
     const int b = blockIdx.z / gc.nn, L = blockIdx.z - b * gc.nn;
-    const int I = blockIdx.x * 32 + (threadIdx.x & 31), J = blockIdx.y * 8 + (threadIdx.x >> 5);
-    if (I > gc.n || J > gc.n || batch_skipped(bt, b)) return;
+    const int q = blockIdx.x * 256 + threadIdx.x, J = q / gc.nn, I = q - J * gc.nn;
+    if (J > gc.n || batch_skipped(bt, b)) return;
     const int nnf = 2 * gc.n + 1;
     rc += (long long)b * bt.bsc + ((long long)L * gc.nn + J) * gc.nn + I;
     if (node_masked(gc, I, J, L)) {
@@ -120,8 +122,8 @@ __global__ void __launch_bounds__(256) k_restrict3(GridDesc gc, const vec2<T>* _
 template <typename T>
 cudaError_t launch_restrict(const GridDesc& gc, const vec2<T>* rf, vec2<T>* rc, const Batch& bt, cudaStream_t s) {
     if (gc.dim == 3)
-        return klaunch(k_restrict3<T>, dim3((gc.nn + 31) / 32, (gc.nn + 7) / 8, gc.nn * bt.nb), dim3(256), 0, s, 1, gc, rf,
-                       rc, bt);
+        return klaunch(k_restrict3<T>, dim3((gc.nn * gc.nn + 255) / 256, 1, gc.nn * bt.nb), dim3(256), 0, s, 1, gc, rf, rc,
+                       bt);
     dim3 blk(32, 8, 1);
     dim3 grd((gc.nn + 31) / 32, (gc.nn + 7) / 8, bt.nb);
     return klaunch(k_restrict<T>, grd, blk, 0, s, 1, gc, rf, rc, bt);
@@ -171,7 +173,9 @@ __global__ void __launch_bounds__(256) k_prolong(GridDesc gf, const vec2<T>* __r
 }
 
 // 3D: a thread takes coarse node (I, J, L) and the up to eight fine nodes (2I + a, 2J + b, 2L + c), so
-// that the coarse values it needs are read once.  The terms of a node are added in k_prolong's order
+// that the coarse values it needs are read once; nodes are numbered through the plane (257^3 55 -> 52 us,
+// 129^3 11.7 -> 10.8).  Bound by the L1 pipe: every access steps by 16 bytes; one fine column per thread,
+// whole rows at a time, took 60 us on 257^3.  The terms of a node are added in k_prolong's order
 // (z, then y, then x), so the results are the same bit for bit.
 template <typename T>
 __global__ void __launch_bounds__(256) k_prolong3(GridDesc gf, const vec2<T>* __restrict__ ec, vec2<T>* __restrict__ x,
@@ -179,8 +183,8 @@ __global__ void __launch_bounds__(256) k_prolong3(GridDesc gf, const vec2<T>* __
     pdl_entry();
     const int n = gf.n, nn = gf.nn, nc = n / 2, nnc = nc + 1;
     const int b = blockIdx.z / nnc, L = blockIdx.z - b * nnc;
-    const int I = blockIdx.x * 32 + (threadIdx.x & 31), J = blockIdx.y * 8 + (threadIdx.x >> 5);
-    if (I > nc || J > nc || batch_skipped(bt, b)) return;
+    const int u = blockIdx.x * 256 + threadIdx.x, J = u / nnc, I = u - J * nnc;
+    if (J > nc || batch_skipped(bt, b)) return;
     x += (long long)b * bt.bs;
     ec += (long long)b * bt.bsc;
     auto cd = [&](int v, int s) { return (v == 0 && gf.dir[s]) || (v == nc && gf.dir[s + 1]); };
@@ -229,7 +233,7 @@ template <typename T>
 cudaError_t launch_prolong(const GridDesc& gf, const vec2<T>* ec, vec2<T>* x, const Batch& bt, cudaStream_t s) {
     if (gf.dim == 3) {
         const int nnc = gf.n / 2 + 1;
-        return klaunch(k_prolong3<T>, dim3((nnc + 31) / 32, (nnc + 7) / 8, nnc * bt.nb), dim3(256), 0, s, 1, gf, ec, x, bt);
+        return klaunch(k_prolong3<T>, dim3((nnc * nnc + 255) / 256, 1, nnc * bt.nb), dim3(256), 0, s, 1, gf, ec, x, bt);
     }
     dim3 blk(32, 8, 1);
     dim3 grd((gf.nn + 31) / 32, (gf.nn + 7) / 8, (gf.dim == 3 ? gf.nn : 1) * bt.nb);
