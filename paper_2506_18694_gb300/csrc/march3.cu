@@ -10,10 +10,11 @@
 // on a face, edge or corner sums its existing neighbours by group (centre; x, y, z faces;
 // xy, xz, yz edges; corners) with the eight weights of its boundary class.
 //
-// Bound by instruction issue and the shared-memory pipe together (257^3 Jacobi sweep: 59 % and
-// 67 % busy).  Complex sums as packed adds and no boundary checks in the output warps took the
-// sweep from 118 to 113 us; tiles off every face (72 % of them there) compiled without any check, to
-// 109 us, and the V-cycle of that grid from 769 to 740.
+// Bound by the shared-memory pipe (257^3 Jacobi sweep: its wavefronts 78 % busy, issue 52 %), then by the
+// loads' latency at 32 warps per SM.  On that sweep and on that grid's V-cycle, us: complex sums as packed
+// adds and no boundary checks in the output warps 118 -> 113; tiles off every face (72 %) compiled without
+// any check 113 -> 109, 769 -> 740; value and x-sum side by side, one 16-byte access for both, 109 -> 107,
+// 703 -> 685 (129^3 HSS step 162 -> 154).
 #include "internal.h"
 
 namespace hh {
@@ -96,6 +97,12 @@ __device__ __forceinline__ void out3(const MArgs<T>& a, const PCoef<T>& cf, cons
     }
 }
 
+// Field value and x-neighbour sum of a node, side by side: one shared-memory access for both (of 16 bytes
+// in complex64).
+template <typename T> struct __align__(16) Pair3 {
+    vec2<T> v, s;
+};
+
 constexpr int kWarps3 = 8;  // y-rows per tile, including the two halo rows
 
 }  // namespace
@@ -114,9 +121,7 @@ __device__ __forceinline__ void march3_tile(const MArgs<T>& a, int b, int bx, in
     const VPtrs<T> v = problem_ptrs(a, b, false);
     constexpr int NP = R + 2;  // planes loaded
     constexpr bool NEEDZ = MODE != M_APPLY;
-    // [warp][plane][lane]: field value and x-neighbour sum
-    vec2<T>* sv = reinterpret_cast<vec2<T>*>(smem_raw);
-    vec2<T>* ss = sv + kWarps3 * NP * 32;
+    Pair3<T>* const sm = reinterpret_cast<Pair3<T>*>(smem_raw);  // [warp][plane][lane]
     const int lane = threadIdx.x & 31;
     const int w = threadIdx.x >> 5;
     const int n = a.g.n, nn = a.g.nn;
@@ -154,8 +159,12 @@ __device__ __forceinline__ void march3_tile(const MArgs<T>& a, int b, int bx, in
 #pragma unroll
     for (int t = 0; t < NP; ++t) {
         xs[t] = shfl_up3(fv[t]) + shfl_dn3(fv[t]);
-        st<T>(sv, (w * NP + t) * 32 + lane, fv[t]);
-        st<T>(ss, (w * NP + t) * 32 + lane, xs[t]);
+        Pair3<T> e;
+        e.v.x = fv[t].re;
+        e.v.y = fv[t].im;
+        e.s.x = xs[t].re;
+        e.s.y = xs[t].im;
+        sm[(w * NP + t) * 32 + lane] = e;
     }
     __syncthreads();
     if (INNER && !out_row) return;
@@ -170,12 +179,11 @@ __device__ __forceinline__ void march3_tile(const MArgs<T>& a, int b, int bx, in
             constexpr int P = 32, Y = NP * 32;
             const long long p = (long long)js * nn + is + l * ps;
             const Cx<T> zq = NEEDZ ? ld<T>(v.z, p) : cx<T>(0, 0);
-            const Win3<T> q3{ld<T>(sv, e), ld<T>(sv, e + P), ld<T>(sv, e + 2 * P),
-                             ld<T>(ss, e), ld<T>(ss, e + P), ld<T>(ss, e + 2 * P),
-                             ld<T>(sv, e - Y) + ld<T>(sv, e + Y), ld<T>(sv, e + P - Y) + ld<T>(sv, e + P + Y),
-                             ld<T>(sv, e + 2 * P - Y) + ld<T>(sv, e + 2 * P + Y),
-                             ld<T>(ss, e - Y) + ld<T>(ss, e + Y), ld<T>(ss, e + P - Y) + ld<T>(ss, e + P + Y),
-                             ld<T>(ss, e + 2 * P - Y) + ld<T>(ss, e + 2 * P + Y)};
+            auto fv1 = [&](int o) { const vec2<T> u = sm[e + o].v; return cx<T>(u.x, u.y); };
+            auto xs1 = [&](int o) { const vec2<T> u = sm[e + o].s; return cx<T>(u.x, u.y); };
+            const Win3<T> q3{fv1(0), fv1(P), fv1(2 * P), xs1(0), xs1(P), xs1(2 * P),
+                             fv1(-Y) + fv1(Y), fv1(P - Y) + fv1(P + Y), fv1(2 * P - Y) + fv1(2 * P + Y),
+                             xs1(-Y) + xs1(Y), xs1(P - Y) + xs1(P + Y), xs1(2 * P - Y) + xs1(2 * P + Y)};
             const bool vd = void1(is, n, a.g.dir[0], a.g.dir[1]) || void1(js, n, a.g.dir[2], a.g.dir[3]);
             out3<T, MODE, false>(a, cf, bw, v, q3, zq, type1(is, n), type1(js, n), l, vd, p);
         }
@@ -184,22 +192,21 @@ __device__ __forceinline__ void march3_tile(const MArgs<T>& a, int b, int bx, in
     if (!out) return;
     const int wm = w - 1, wp = w + 1;
     // rows j-1 + j+1 summed (value and x-sum) per plane, in a rolling window of 3 planes
-    auto ysum = [&](const vec2<T>* arr, int tpl) {
-        return ld<T>(arr, (wm * NP + tpl) * 32 + lane) + ld<T>(arr, (wp * NP + tpl) * 32 + lane);
+    auto ysum = [&](int tpl, Cx<T>& vy, Cx<T>& sy) {
+        const Pair3<T> m = sm[(wm * NP + tpl) * 32 + lane], p = sm[(wp * NP + tpl) * 32 + lane];
+        vy = cx<T>(m.v.x, m.v.y) + cx<T>(p.v.x, p.v.y);
+        sy = cx<T>(m.s.x, m.s.y) + cx<T>(p.s.x, p.s.y);
     };
     Win3<T> q;
-    q.vy0 = ysum(sv, 0);
-    q.vy1 = ysum(sv, 1);
-    q.sy0 = ysum(ss, 0);
-    q.sy1 = ysum(ss, 1);
+    ysum(0, q.vy0, q.sy0);
+    ysum(1, q.vy1, q.sy1);
     const long long p0 = col;
 #pragma unroll
     for (int t = 0; t < R; ++t) {
         const int l = l0 + t;
         if (!INNER && l > n) break;
         const int tp = t + 1;  // local plane of the output
-        q.vy2 = ysum(sv, tp + 1);
-        q.sy2 = ysum(ss, tp + 1);
+        ysum(tp + 1, q.vy2, q.sy2);
         q.fm = fv[tp - 1];
         q.f0 = fv[tp];
         q.fp = fv[tp + 1];
