@@ -322,7 +322,7 @@ static int g_fit_size3 = 0;  // cluster size that decides which 3D levels run in
 int coarse_cluster_size() {
     if (g_cluster_size) return g_cluster_size;
     cudaFuncAttributes fa = {};
-    const bool single_only = cudaFuncGetAttributes(&fa, k_coarse_dsmem<float, 2>) != cudaSuccess ||
+    const bool float_unprepared = cudaFuncGetAttributes(&fa, k_coarse_dsmem<float, 2>) != cudaSuccess ||
                              fa.maxDynamicSharedSizeBytes < (int)kCoarseSmemMax;
     cudaGetLastError();
     // the query below asks for kCoarseSmemMax, which the queried kernel has to be allowed: where only the
@@ -349,7 +349,7 @@ int coarse_cluster_size() {
     cfg.numAttrs = 1;
     int nclusters = 0;
     if (cudaOccupancyMaxActiveClusters(&nclusters, k_coarse_dsmem<float, 2>, &cfg) == cudaSuccess && nclusters >= 1) {
-        g_fit_size3 = single_only ? 1 : cs;
+        g_fit_size3 = float_unprepared ? 1 : cs;
         g_cluster_size = cs;
         return cs;
     }

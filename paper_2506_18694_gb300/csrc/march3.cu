@@ -10,7 +10,7 @@
 // on a face, edge or corner sums its existing neighbours by group (centre; x, y, z faces;
 // xy, xz, yz edges; corners) with the eight weights of its boundary class.
 //
-// Bound by the shared-memory pipe (257^3 Jacobi sweep: its wavefronts 78 % busy, issue 52 %), then by the
+// Bound by the shared-memory pipe (257^3 Jacobi sweep: its wavefronts 76 % busy, issue 52 %), then by the
 // loads' latency at 32 warps per SM.  On that sweep and on that grid's V-cycle, us: complex sums as packed
 // adds and no boundary checks in the output warps 118 -> 113; tiles off every face (72 %) compiled without
 // any check 113 -> 109, 769 -> 740; value and x-sum side by side, one 16-byte access for both, 109 -> 107,
