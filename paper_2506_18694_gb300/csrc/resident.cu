@@ -25,7 +25,9 @@
 // at most one pass ahead, because it needs our rows, and each of our threads that reads a halo row
 // sends its result to the same neighbour after that read.  The right side of the first replicated
 // level goes to every CTA by bulk copies; a split cluster barrier (arrive after the replicated
-// levels, wait before the next copies) keeps them from overwriting one in use.  Every wait is
+// levels, wait before the next right side's first store) keeps a CTA from overwriting rows that a
+// copy to a CTA far away may still be reading, and its copies from overwriting one in use: halo
+// exchanges hold back adjacent CTAs only, a CTA six rows of them away can be a step behind.  Every wait is
 // bounded (spin_limit polls): a CTA that gives up skips the rest of its passes, but not the cluster
 // barriers; its neighbours' waits run out in turn, and the launch ends with HH_ERR_TIMEOUT recorded.
 //
@@ -481,10 +483,9 @@ __device__ __noinline__ void restrict_pass(const Res S, int lvl, int copies) {
     Head<T>& hd = head<T>();
     const Lev L = hd.lv[lvl], M = hd.lv[lvl + 1];
     const bool spread = M.rep && !L.rep && S.cs > 1;  // the level's right side goes to every CTA
-    if (hd.dead) {
-        if (spread) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-        return;
-    }
+    // every CTA is done with the last right side, ours (whose rows the loop below overwrites) included
+    if (spread) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (hd.dead) return;
     const PCoef<T>& c = hd.coef[lvl + 1];
     vec2<T>* const sm = vecs<T>();
     const Push ps = push_rows<T>(S, M, M.A);
@@ -522,10 +523,9 @@ __device__ __noinline__ void restrict_pass(const Res S, int lvl, int copies) {
         pass_end<T>(S, M);
         return;
     }
-    // our rows of the right side to every other CTA, once all are done with the previous one
+    // our rows of the right side to every other CTA
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     if ((int)threadIdx.x < S.cs && (int)threadIdx.x != S.rank && M.bulkn > 0) {
         const unsigned src = saddr(sm + M.b + M.bulk0 * M.W), bytes = (unsigned)(M.bulkn * M.W * sizeof(vec2<T>));
         asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
