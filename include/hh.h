@@ -66,7 +66,7 @@ typedef enum {
     HH_ERR_OOM = -2,        /* device allocation failed                               */
     HH_ERR_CUDA = -3,       /* a CUDA runtime call failed                             */
     HH_ERR_NONFINITE = -4,  /* NaN or Inf met in the right side or the iteration      */
-    HH_ERR_TIMEOUT = -5     /* a bounded device wait (grid-wide barrier) ran out      */
+    HH_ERR_TIMEOUT = -5     /* a bounded wait inside a kernel ran out                */
 } hh_status;
 
 /* Boundary tags of Sec. 1: Gamma (radiation condition) and dOmega_0 (u = 0). */
@@ -157,9 +157,11 @@ typedef struct {
                          /* kernel whose CTAs meet at grid-wide barriers between the passes of */
                          /* each cycle; 2: at every size; 0 (default): one kernel per pass,    */
                          /* replayed from a CUDA graph.  Same result bit for bit               */
-    long long sync_spin_limit; /* polls a grid-wide barrier wait may take before the kernel     */
-                         /* gives up and the call returns HH_ERR_TIMEOUT; 0 = 4194304 (about   */
-                         /* a second or more); tiny values make the waits run out on purpose   */
+    long long sync_spin_limit; /* polls a wait inside a kernel (of the persistent loop at its grid-wide */
+                         /* barriers, of the one-cluster loop or cycle of a small 2D problem for */
+                         /* its neighbours' rows) may take before the kernel gives up and the    */
+                         /* call returns HH_ERR_TIMEOUT; 0 = 4194304; tiny values make the waits */
+                         /* run out on purpose                                                   */
     int stall_cycles;    /* > 0: FGMRES gives a problem up (HH_NOT_CONVERGED, last iterate in u) */
                          /* when stall_cycles restart cycles in a row did not halve its true    */
                          /* residual; 0 (default): only max_outer ends it                       */

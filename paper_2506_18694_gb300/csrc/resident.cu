@@ -27,9 +27,14 @@
 // level goes to every CTA by bulk copies; a split cluster barrier (arrive after the replicated
 // levels, wait before the next right side's first store) keeps a CTA from overwriting rows that a
 // copy to a CTA far away may still be reading, and its copies from overwriting one in use: halo
-// exchanges hold back adjacent CTAs only, a CTA six rows of them away can be a step behind.  Every wait is
-// bounded (spin_limit polls): a CTA that gives up skips the rest of its passes, but not the cluster
-// barriers; its neighbours' waits run out in turn, and the launch ends with HH_ERR_TIMEOUT recorded.
+// exchanges hold back adjacent CTAs only, a CTA six rows of them away can be a step behind.
+//
+// Every wait is bounded (spin_limit polls): a CTA that gives up skips the rest of its passes, but not
+// the cluster barriers; its neighbours' waits run out in turn, and the launch ends with HH_ERR_TIMEOUT
+// recorded.  That a wait ran out is read by every thread behind the pass's block barrier, from a word that
+// is not written again before the next one, so the whole CTA gives up at the same pass.  What others
+// sent to a CTA that gave up is still on its way when the passes end: the CTAs of such a cluster tell
+// one another how many passes and copies they sent, and each waits for its own (give_up).
 //
 // Work split of a pass: complex64, a thread takes two neighbouring columns (one 16-byte and two
 // 8-byte shared loads per row) and 1, 2 or 4 rows; complex128, two lanes take the real and the
@@ -87,14 +92,16 @@ __device__ __forceinline__ int kind_of(unsigned d) { return (d >> 22) & 15; }  /
 enum { P_SWEEP = 0, P_RESID = 1, P_HSS = 2, P_FIRST = 3 };  // P_FIRST: the first sweep from 0
 
 // Start of the dynamic shared memory: coefficients of the levels and of the HSS step (index
-// levels), the levels, the halo barriers [from above, from below][alternating] and the one of the
-// replicated right side, the give-up flag; then the level vectors (at kHead<T> bytes).
+// levels), the levels, the halo barriers [from above, from below][alternating] and those of the
+// replicated right side [alternating], whether a wait of a halo exchange [alternating] or of the right
+// side [2] ran out; for a cluster in which one did: that it did, the passes and right sides this CTA
+// sent, and the bytes of a halo row of its last pass.  Then the level vectors (at kHead<T> bytes).
 template <typename T> struct Head {
     PCoef<T> coef[kResMaxLevels + 1];
     Lev lv[kResMaxLevels];
     unsigned long long mb[2][2];
-    unsigned long long mbr;
-    int dead;
+    unsigned long long mbr[2];
+    int gave_up[3], any, rounds, copies, row_bytes;
 };
 template <typename T> constexpr size_t kHead = (sizeof(Head<T>) + 127) / 128 * 128;
 
@@ -145,12 +152,15 @@ __device__ __forceinline__ bool bar_try(unsigned bar, unsigned parity) {
 }
 
 // The cluster as a CTA sees it: Dirichlet sides (bit s: side s), the level vectors' address in the
-// CTAs above and below, and the number of passes that ended with a halo exchange.
+// CTAs above and below, and the number of passes that exchanged halo rows, with kDead set when a wait
+// of this CTA ran out: its later passes do nothing.
+constexpr int kDead = 1 << 30;
 struct Res {
     int rank, cs, dir;
     unsigned base_up, base_dn, mb_up, mb_dn;  // (mb_*: the neighbour's barrier of what we send)
     int round;
     unsigned long long spin;
+    __device__ __forceinline__ bool dead() const { return round & kDead; }
 };
 
 // Where a pass sends its first and last row: the addresses that, with the node's own offset in the
@@ -164,22 +174,17 @@ __device__ __forceinline__ Push push_rows(const Res& S, const Lev& L, int buf) {
     return Push{S.base_up + (buf + L.Ru * L.W) * e, S.base_dn + (buf - L.R * L.W) * e, S.mb_up + k, S.mb_dn + k};
 }
 
-// Wait for a barrier's phase, at most `spin` polls; then the CTA has given up (called before a block
-// barrier: every thread sees the flag at the next pass).
-template <typename T>
-__device__ __forceinline__ void bounded_wait(unsigned long long* bar, unsigned parity, unsigned long long spin) {
-    Head<T>& hd = head<T>();
+// Wait for a barrier's phase, at most `spin` polls; false when they run out.
+__device__ __forceinline__ bool bounded_wait(unsigned long long* bar, unsigned parity, unsigned long long spin) {
     unsigned long long k = 0;
-    while (!bar_try(saddr(bar), parity)) {
-        if (++k > spin) {
-            hd.dead = 1;
-            return;
-        }
-    }
+    while (!bar_try(saddr(bar), parity))
+        if (++k > spin) return false;
+    return true;
 }
 
 // End of a pass whose first and last rows were sent: thread 0 waits for the row from above, thread
-// 32 for the one from below, then the block meets.  (pass_begin: what the pass expects.)
+// 32 for the one from below, then the block meets and sees whether a wait ran out.  The next pass that
+// writes the same word comes after one more block barrier.  (pass_begin: what the pass expects.)
 template <typename T>
 __device__ __forceinline__ void pass_begin(const Res& S, const Lev& L) {
     Head<T>& hd = head<T>();
@@ -188,11 +193,17 @@ __device__ __forceinline__ void pass_begin(const Res& S, const Lev& L) {
     if (threadIdx.x == 32 && L.dn) bar_expect(saddr(&hd.mb[1][S.round & 1]), bytes);
 }
 template <typename T>
-__device__ __forceinline__ void pass_end(const Res& S, const Lev& L) {
+__device__ __forceinline__ void pass_end(Res& S, const Lev& L) {
     Head<T>& hd = head<T>();
-    if (threadIdx.x == 0 && L.up) bounded_wait<T>(&hd.mb[0][S.round & 1], (S.round >> 1) & 1, S.spin);
-    if (threadIdx.x == 32 && L.dn) bounded_wait<T>(&hd.mb[1][S.round & 1], (S.round >> 1) & 1, S.spin);
+    const int k = S.round & 1, d = threadIdx.x == 0 ? 0 : 1;
+    if ((threadIdx.x == 0 && L.up) || (threadIdx.x == 32 && L.dn)) {
+        if (!bounded_wait(&hd.mb[d][k], (S.round >> 1) & 1, S.spin)) {
+            hd.gave_up[k] = kDead;
+            hd.row_bytes = L.nn * (int)sizeof(vec2<T>);
+        }
+    }
     __syncthreads();
+    S.round = (S.round + 1) | hd.gave_up[k];
 }
 
 __device__ __forceinline__ void st_pair(float2* p, Cx<float> a, Cx<float> b) {
@@ -443,7 +454,6 @@ __device__ __forceinline__ void run(Res& S, const Lev& L, const PCoef<T>& c, con
         __syncthreads();
     } else {
         pass_end<T>(S, L);
-        ++S.round;
     }
 }
 
@@ -453,21 +463,21 @@ __device__ __forceinline__ void run_two(Res& S, const Lev& L, const PCoef<T>& c,
     const Mine<T> m = mine<T, FIRST>(L, c);
     run<T, FIRST, TR, REP>(S, L, c, m, src, dst, bsrc);
     if constexpr (SECOND >= 0) {
-        if (!REP && head<T>().dead) return;
+        if (!REP && S.dead()) return;
         run<T, SECOND, TR, REP>(S, L, c, m, dst, src, bsrc);
     }
 }
 
-// The same for level `lvl` with coefficient record `ci`; returns the rounds of halo exchanges so far.
+// The same for level `lvl` with coefficient record `ci`; returns S.round.
 template <typename T, int FIRST, int SECOND>
 __device__ __noinline__ int passes(Res S, int lvl, int ci, int src, int dst, int bsrc) {
+    if (S.dead()) return S.round;
     const Lev L = head<T>().lv[lvl];
     const PCoef<T>& c = head<T>().coef[ci];
     if (L.rep) {
         if (sizeof(T) == 8 || L.tr == 1) run_two<T, FIRST, SECOND, 1, true>(S, L, c, src, dst, bsrc);
         else run_two<T, FIRST, SECOND, 4, true>(S, L, c, src, dst, bsrc);
     } else {
-        if (head<T>().dead) return S.round;
         if (sizeof(T) == 8 || L.tr == 1) run_two<T, FIRST, SECOND, 1, false>(S, L, c, src, dst, bsrc);
         else if (L.tr == 2) run_two<T, FIRST, SECOND, 2, false>(S, L, c, src, dst, bsrc);
         else run_two<T, FIRST, SECOND, 4, false>(S, L, c, src, dst, bsrc);
@@ -479,19 +489,19 @@ __device__ __noinline__ int passes(Res S, int lvl, int ci, int src, int dst, int
 // level's first sweep from 0 into its A.  `copies`: the number of right sides sent to the
 // replicated levels so far.
 template <typename T>
-__device__ __noinline__ void restrict_pass(const Res S, int lvl, int copies) {
+__device__ __noinline__ int restrict_pass(Res S, int lvl, int copies) {
     Head<T>& hd = head<T>();
     const Lev L = hd.lv[lvl], M = hd.lv[lvl + 1];
     const bool spread = M.rep && !L.rep && S.cs > 1;  // the level's right side goes to every CTA
     // every CTA is done with the last right side, ours (whose rows the loop below overwrites) included
     if (spread) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    if (hd.dead) return;
+    if (S.dead()) return S.round;
     const PCoef<T>& c = hd.coef[lvl + 1];
     vec2<T>* const sm = vecs<T>();
     const Push ps = push_rows<T>(S, M, M.A);
     pass_begin<T>(S, M);
     if (spread && threadIdx.x == 0)
-        bar_expect(saddr(&hd.mbr), (unsigned)((M.nn - M.bulkn) * M.W * sizeof(vec2<T>)));
+        bar_expect(saddr(&hd.mbr[copies & 1]), (unsigned)((M.nn - M.bulkn) * M.W * sizeof(vec2<T>)));
     const uint2* dw = reinterpret_cast<const uint2*>(words<T>() + M.r0);
     for (int it = threadIdx.x; it < M.restricted; it += kResThreads) {
         // x: offset of fine node (2I, 2J - 1) in A, and of coarse node (I, J) in an iterate << 16
@@ -520,8 +530,9 @@ __device__ __noinline__ void restrict_pass(const Res S, int lvl, int copies) {
         if (d.y & kDn) send(ps.dn + at * (unsigned)sizeof(vec2<T>), x1, ps.bdn);
     }
     if (!spread) {
-        pass_end<T>(S, M);
-        return;
+        if (M.rep) __syncthreads();
+        else pass_end<T>(S, M);
+        return S.round;
     }
     // our rows of the right side to every other CTA
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -530,11 +541,12 @@ __device__ __noinline__ void restrict_pass(const Res S, int lvl, int copies) {
         const unsigned src = saddr(sm + M.b + M.bulk0 * M.W), bytes = (unsigned)(M.bulkn * M.W * sizeof(vec2<T>));
         asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                          remote(src, threadIdx.x)),
-                     "r"(src), "r"(bytes), "r"(remote(saddr(&hd.mbr), threadIdx.x))
+                     "r"(src), "r"(bytes), "r"(remote(saddr(&hd.mbr[copies & 1]), threadIdx.x))
                      : "memory");
     }
-    if (threadIdx.x == 0) bounded_wait<T>(&hd.mbr, copies & 1, S.spin);
+    if (threadIdx.x == 0 && !bounded_wait(&hd.mbr[copies & 1], (copies >> 1) & 1, S.spin)) hd.gave_up[2] = kDead;
     __syncthreads();
+    return S.round | hd.gave_up[2];
 }
 
 // The coarsest level: its first sweep is in A, the last one has to end in B.
@@ -546,11 +558,12 @@ __device__ __forceinline__ void sweeps(Res& S, const Lev& L, const PCoef<T>& c, 
         const int t = src;
         src = dst;
         dst = t;
-        if (!REP && head<T>().dead) return;
+        if (!REP && S.dead()) return;
     }
 }
 template <typename T>
 __device__ __noinline__ int coarse_sweeps(Res S, int lvl, int nsweeps) {
+    if (S.dead()) return S.round;
     const Lev L = head<T>().lv[lvl];
     const PCoef<T>& c = head<T>().coef[lvl];
     int src = L.A, dst = L.B;
@@ -558,7 +571,6 @@ __device__ __noinline__ int coarse_sweeps(Res S, int lvl, int nsweeps) {
         if (sizeof(T) == 8 || L.tr == 1) sweeps<T, 1, true>(S, L, c, nsweeps, src, dst);
         else sweeps<T, 4, true>(S, L, c, nsweeps, src, dst);
     } else {
-        if (head<T>().dead) return S.round;
         if (sizeof(T) == 8 || L.tr == 1) sweeps<T, 1, false>(S, L, c, nsweeps, src, dst);
         else if (L.tr == 2) sweeps<T, 2, false>(S, L, c, nsweeps, src, dst);
         else sweeps<T, 4, false>(S, L, c, nsweeps, src, dst);
@@ -574,7 +586,7 @@ __device__ __noinline__ int coarse_sweeps(Res S, int lvl, int nsweeps) {
 // B of level lvl += P e, e the iterate in B of level lvl + 1, on our rows and the halo rows
 template <typename T>
 __device__ __noinline__ void prolong_pass(const Res S, int lvl) {
-    if (head<T>().dead) return;
+    if (S.dead()) return;
     const Lev& L = head<T>().lv[lvl];
     const Lev& M = head<T>().lv[lvl + 1];
     vec2<T>* const sm = vecs<T>();
@@ -598,6 +610,56 @@ __device__ __noinline__ void prolong_pass(const Res S, int lvl) {
         if (d.y & 8) st<T>(x, 1, x3 + half_rn(c10 + c11));
     }
     __syncthreads();
+}
+
+// A value of another CTA's shared memory, at the address of our own copy.
+__device__ __forceinline__ int peer(const int* p, int rank) {
+    int v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(remote(saddr(p), rank)) : "memory");
+    return v;
+}
+
+// A cluster in which a wait ran out, after the cluster barrier behind its passes (every CTA has sent what it
+// will): a CTA that gave up waits for what is still on its way to it, so that none of it arrives after the
+// CTA has left.  Of the halo rows that is its last pass's, if the neighbour sent them, and those of one
+// pass more, in which the neighbour gave up for want of our rows (hence its row_bytes); of the right
+// sides (`copies` sent here so far, level lr) the last one's from the CTAs that sent it, and the next one's.
+template <typename T>
+__device__ __noinline__ void give_up(const Res S, int copies, int lr) {
+    Head<T>& hd = head<T>();
+    constexpr unsigned long long kDrain = 4194304;  // (microseconds are enough)
+    const int r = S.round & ~kDead;
+    if ((threadIdx.x == 0 && S.rank > 0) || (threadIdx.x == 32 && S.rank + 1 < S.cs)) {
+        const int d = threadIdx.x == 0 ? 0 : 1, q = S.rank + 2 * d - 1;
+        const int sent = peer(&hd.rounds, q);
+        if (r > 0 && sent >= r) bounded_wait(&hd.mb[d][(r - 1) & 1], ((r - 1) >> 1) & 1, kDrain);
+        if (sent > r) {
+            bar_expect(saddr(&hd.mb[d][r & 1]), (unsigned)peer(&hd.row_bytes, q));
+            bounded_wait(&hd.mb[d][r & 1], (r >> 1) & 1, kDrain);
+        }
+    }
+    if (threadIdx.x == 64 && lr > 0) {
+        unsigned missing = 0, next = 0;
+        for (int q = 0; q < S.cs; ++q) {
+            if (q == S.rank) continue;
+            const unsigned bytes = (unsigned)(peer(&hd.lv[lr].bulkn, q) * hd.lv[lr].W * (int)sizeof(vec2<T>));
+            const int sent = peer(&hd.copies, q);
+            if (sent < copies) missing += bytes;
+            if (sent > copies) next += bytes;
+        }
+        if (copies > 0) {
+            unsigned long long* bar = &hd.mbr[(copies - 1) & 1];
+            if (missing)
+                asm volatile("mbarrier.complete_tx.relaxed.cluster.shared::cta.b64 [%0], %1;" ::"r"(saddr(bar)),
+                             "r"(missing)
+                             : "memory");
+            bounded_wait(bar, ((copies - 1) >> 1) & 1, kDrain);
+        }
+        if (next) {
+            bar_expect(saddr(&hd.mbr[copies & 1]), next);
+            bounded_wait(&hd.mbr[copies & 1], (copies >> 1) & 1, kDrain);
+        }
+    }
 }
 
 // ---- set-up: the levels and their item words ----
@@ -772,9 +834,10 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident2(const __grid_const
     if (threadIdx.x == 0) {
         for (int q = 0; q < 4; ++q)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&hd.mb[q >> 1][q & 1])) : "memory");
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&hd.mbr)) : "memory");
+        for (int q = 0; q < 2; ++q)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&hd.mbr[q])) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        hd.dead = 0;
+        hd.gave_up[0] = hd.gave_up[1] = hd.gave_up[2] = hd.any = 0;
     } else if (threadIdx.x == 32) {
         const int nn0 = a.lv[0].nn;
         int f0 = S.rank * nn0 / a.cs, f1 = (S.rank + 1) * nn0 / a.cs, fu = S.rank > 0 ? (S.rank - 1) * nn0 / a.cs : 0;
@@ -818,6 +881,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident2(const __grid_const
     if (copies) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 
     const int steps = HSS ? a.nhss[prob] : 1;
+    int sent = 0;  // right sides sent to the other CTAs
     for (int it = 0; it < steps; ++it) {
         if (HSS) {
             if (!keep) {
@@ -833,8 +897,8 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident2(const __grid_const
         }
         for (int l = 0; l < Lc - 1; ++l) {
             S.round = passes<T, P_SWEEP, P_RESID>(S, l, l, hd.lv[l].A, hd.lv[l].B, hd.lv[l].b);
-            restrict_pass<T>(S, l, it);
-            S.round += l + 1 < a.dist;
+            if (!S.dead() && l + 1 == a.dist) sent = it + 1;
+            S.round = restrict_pass<T>(S, l, it);
             if (copies && l + 1 == a.dist)
                 passes<T, P_FIRST, -1>(S, l + 1, l + 1, hd.lv[l + 1].A, hd.lv[l + 1].A, hd.lv[l + 1].b);
         }
@@ -855,8 +919,20 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident2(const __grid_const
         else
             st<T>(a.x, base + q, v);
     }
-    if (threadIdx.x == 0 && hd.dead) *a.status = -5;  // HH_ERR_TIMEOUT
-    if (a.cs > 1) cg::this_cluster().sync();  // nobody leaves while another may still send to it
+    if (a.cs == 1) return;
+    if (threadIdx.x == 0) {
+        hd.rounds = S.round & ~kDead;
+        hd.copies = sent;
+        if (S.dead()) *a.status = -5;  // HH_ERR_TIMEOUT
+    }
+    if (S.dead() && (int)threadIdx.x < S.cs)
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote(saddr(&hd.any), threadIdx.x)), "r"(1) : "memory");
+    cg::this_cluster().sync();  // nobody leaves while another may still send to it
+    if (hd.any) {
+        if (S.dead()) give_up<T>(S, sent, copies ? a.dist : 0);
+        __syncthreads();
+        cg::this_cluster().sync();
+    }
 }
 
 namespace {

@@ -1137,7 +1137,7 @@ hh::ResArgs<T>* resident(hh_problem* p, bool hss) {
             P.nhss = p->d_nhss;
             P.active = active_flags(p);
             P.status = (int*)(p->d_sync + 1);
-            P.spin_limit = 4194304ULL;  // (sync_spin_limit is the persistent loop's)
+            P.spin_limit = p->o.sync_spin_limit > 0 ? (unsigned long long)p->o.sync_spin_limit : 4194304ULL;
             H.res[hss].resize(sizeof(P));
             std::memcpy(H.res[hss].data(), &P, sizeof(P));
             H.res_state[hss] = 1;
@@ -1459,16 +1459,17 @@ hh_status norm2_dev(hh_problem* p, const double2* v, int slot) {
     return HH_OK;
 }
 
-// The status word of the persistent HSS loop (copied with every fetch): a non-zero value is
-// an error a CTA recorded; it is cleared here and returned.
+// The status word of the kernels with bounded waits (the persistent HSS loop, the cluster-resident
+// loops and cycles), copied with every fetch: a non-zero value is an error a CTA recorded; it is cleared
+// here and returned.
 hh_status check_sync(hh_problem* p) {
     const int st = *p->h_sync;
     if (st == 0) return HH_OK;
     *p->h_sync = 0;
     HH_CUDA(cudaMemsetAsync(p->d_sync + 1, 0, sizeof(int), p->s));
     HH_CUDA(cudaStreamSynchronize(p->s));
-    return fail((hh_status)st, st == HH_ERR_TIMEOUT ? "a grid-wide barrier wait of the persistent HSS loop ran out"
-                                                    : "the persistent HSS loop reported an error");
+    return fail((hh_status)st, st == HH_ERR_TIMEOUT ? "a bounded device wait of the HSS loop or cycle ran out"
+                                                    : "the HSS loop reported an error");
 }
 
 hh_status fetch(hh_problem* p) {
