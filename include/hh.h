@@ -327,7 +327,9 @@ HH_API hh_status hh_residual_restrict(hh_problem* p, int level, int precision, c
 HH_API hh_status hh_prolong_correct(hh_problem* p, int level, int precision, const void* ec, void* x);
 
 /* x = one multigrid cycle (V or W, cycle_gamma) on A_L of level 0 from the zero initial guess
- * (cycles_per_hss ignored). */
+ * (cycles_per_hss ignored).  Non-blocking, also where a wait inside its kernel runs out
+ * (sync_spin_limit): x of that problem is then NaN throughout, and the next hh_prepare,
+ * hh_precondition or solve of the problem object returns HH_ERR_TIMEOUT. */
 HH_API hh_status hh_vcycle(hh_problem* p, int precision, const void* b, void* x);
 
 /* rhs = (k-1)/(k+1) A_R u + 2k/(k+1) r on level 0 (Def. 4.1); u == NULL means u = 0. */

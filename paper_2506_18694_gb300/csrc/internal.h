@@ -295,6 +295,7 @@ cudaError_t launch_pack_pass(int kind, const HssLoop2<T>* plans, const int* star
 // V(2,2) scaled-Jacobi cycles on `levels` levels, every level vector in distributed shared memory
 // (lv: its offsets); levels from `dist` on are held whole by every CTA.
 constexpr int kResMaxLevels = 6;
+constexpr int kLoopTimeout = -5, kCycleTimeout = -105;  // status: HH_ERR_TIMEOUT, of an HSS loop or of one cycle
 struct ResLevel {
     int nn, W, offA, offB, offb, offt, offr, offp;
 };
@@ -311,7 +312,7 @@ template <typename T> struct ResArgs {
     int nu_coarse;
     const int* nhss;
     const int* active;
-    int* status;  // set to HH_ERR_TIMEOUT when a wait ran past spin_limit polls
+    int* status;  // set to kLoopTimeout or kCycleTimeout when a wait ran past spin_limit polls
     unsigned long long spin_limit;
     const double2* r;  // HSS loop: input and result, and a vector of the problem for r in T
     double2* z;

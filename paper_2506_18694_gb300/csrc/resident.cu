@@ -30,8 +30,8 @@
 // exchanges hold back adjacent CTAs only, a CTA six rows of them away can be a step behind.
 //
 // Every wait is bounded (spin_limit polls): a CTA that gives up skips the rest of its passes, but not
-// the cluster barriers; its neighbours' waits run out in turn, and the launch ends with HH_ERR_TIMEOUT
-// recorded.  That a wait ran out is read by every thread behind the pass's block barrier, from a word that
+// the cluster barriers; its neighbours' waits run out in turn, and the launch ends with the status
+// recorded and a result of NaN.  That a wait ran out is read by every thread behind the pass's block barrier, from a word that
 // is not written again before the next one, so the whole CTA gives up at the same pass.  What others
 // sent to a CTA that gave up is still on its way when the passes end: the CTAs of such a cluster tell
 // one another how many passes and copies they sent, and each waits for its own (give_up).
@@ -911,25 +911,29 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident2(const __grid_const
         }
     }
     if (copies) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    auto write = [&](long long p, Cx<T> v) {
+        if constexpr (HSS)
+            a.z[p] = make_double2((double)v.re, (double)v.im);
+        else
+            st<T>(a.x, p, v);
+    };
     for (int q = threadIdx.x; q < L0.R * nn0; q += kResThreads) {
         const int rl = q / nn0, i = q - rl * nn0;
-        const Cx<T> v = ld<T>(sm, L0.B + (rl + 1) * L0.W + i + 1);
-        if constexpr (HSS)
-            a.z[base + q] = make_double2((double)v.re, (double)v.im);
-        else
-            st<T>(a.x, base + q, v);
+        write(base + q, ld<T>(sm, L0.B + (rl + 1) * L0.W + i + 1));
     }
     if (a.cs == 1) return;
     if (threadIdx.x == 0) {
         hd.rounds = S.round & ~kDead;
         hd.copies = sent;
-        if (S.dead()) *a.status = -5;  // HH_ERR_TIMEOUT
+        if (S.dead()) *a.status = HSS ? kLoopTimeout : kCycleTimeout;
     }
     if (S.dead() && (int)threadIdx.x < S.cs)
         asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote(saddr(&hd.any), threadIdx.x)), "r"(1) : "memory");
     cg::this_cluster().sync();  // nobody leaves while another may still send to it
     if (hd.any) {
         if (S.dead()) give_up<T>(S, sent, copies ? a.dist : 0);
+        // no half-finished result: a single cycle's caller is told only by its next blocking call
+        for (int q = threadIdx.x; q < L0.R * nn0; q += kResThreads) write(base + q, cx<T>(T(NAN), T(NAN)));
         __syncthreads();
         cg::this_cluster().sync();
     }

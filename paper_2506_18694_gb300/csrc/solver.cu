@@ -1468,7 +1468,10 @@ hh_status check_sync(hh_problem* p) {
     *p->h_sync = 0;
     HH_CUDA(cudaMemsetAsync(p->d_sync + 1, 0, sizeof(int), p->s));
     HH_CUDA(cudaStreamSynchronize(p->s));
-    return fail((hh_status)st, st == HH_ERR_TIMEOUT ? "a bounded device wait of the HSS loop or cycle ran out"
+    // (the cycle's own call did not block)
+    if (st == hh::kCycleTimeout)
+        return fail(HH_ERR_TIMEOUT, "a bounded device wait of an earlier hh_vcycle of this problem ran out: its result is NaN");
+    return fail((hh_status)st, st == HH_ERR_TIMEOUT ? "a bounded device wait of the HSS loop ran out"
                                                     : "the HSS loop reported an error");
 }
 
