@@ -805,7 +805,10 @@ __device__ void make_words(const ResArgs<T>& a, const Res& S, int l) {
 // (complex128 in and out); else x = one cycle on A_L x = b from 0 (vectors in T).
 template <typename T, bool HSS>
 __global__ void __launch_bounds__(kResThreads, 1) k_resident2(const __grid_constant__ ResArgs<T> a) {
-    pdl_entry();
+    // (the kernels behind this one may not come before its end: parked on the free SMs for the length of an HSS
+    // loop, their blocks kept the clusters of other streams, which want 16 SMs to themselves, from starting.
+    // 48 uneven solves per second on four worker slots / in one pack: 15.9 / 34.4 so, 33.6 / 57.5 now)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int prob = blockIdx.x / a.cs;
     if (a.active && !a.active[prob]) return;  // uniform over the cluster
     Head<T>& hd = head<T>();
@@ -911,6 +914,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident2(const __grid_const
         }
     }
     if (copies) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     auto write = [&](long long p, Cx<T> v) {
         if constexpr (HSS)
             a.z[p] = make_double2((double)v.re, (double)v.im);
