@@ -12,6 +12,8 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <atomic>
+#include <mutex>
 
 #include "internal.h"
 #include "march2_common.cuh"
@@ -64,8 +66,8 @@ static SlabPlan slab_plan(const GridDesc& g, int cs) {
 // K nodes per thread; a sweep lasts as long as one warp's chain over them (nodes near a side take about
 // 400 instructions), so K = 1 wherever the CTA's nodes allow, with the 1D rows kept over the sweeps, and
 // the cluster is the smallest that gives each thread a node (fewer CTAs to wait for).  HSS step with the
-// coarsest level 3^3, 5^3, 6^3, 17^3, us: 48.2 -> 43.7, 51.6 -> 46.1, 52.6 -> 48.5, 172 -> 164.
-constexpr int kCoarseThreads1 = 640;  // K = 1: holds two planes of 17^2
+// coarsest level 3^3, 5^3, 6^3, us: 48.2 -> 43.7, 51.6 -> 46.1, 52.6 -> 48.5.
+constexpr int kCoarseThreads1 = 640;
 template <typename T, int K>
 __global__ void __launch_bounds__(K == 1 ? kCoarseThreads1 : kCoarseThreads)
 k_coarse_dsmem(const __grid_constant__ MArgs<T> a, int nsweeps, int per) {
@@ -316,16 +318,9 @@ static int band_rows(const GridDesc& g, int nsweeps, int want) {
     return band2_smem<T>(g.nn, nsweeps, R) <= kCoarseSmemMax ? R : 0;
 }
 
-static int g_cluster_size = 0;
-static int g_fit_size3 = 0;  // cluster size that decides which 3D levels run in a cluster (coarse_fits)
-
-int coarse_cluster_size() {
-    if (g_cluster_size) return g_cluster_size;
-    cudaFuncAttributes fa = {};
-    const bool float_unprepared = cudaFuncGetAttributes(&fa, k_coarse_dsmem<float, 2>) != cudaSuccess ||
-                             fa.maxDynamicSharedSizeBytes < (int)kCoarseSmemMax;
-    cudaGetLastError();
-    // the query below asks for kCoarseSmemMax, which the queried kernel has to be allowed: where only the
+// The largest of 16 and 8 CTAs whose cluster the current device holds, else 1.
+static int query_cluster_size() {
+    // the query asks for kCoarseSmemMax, which the queried kernel has to be allowed: where only the
     // complex128 kernels had been prepared it failed and the level ran in one CTA (33^2: 128 us)
     cudaFuncSetAttribute(k_coarse_dsmem<float, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmemMax);
     cudaFuncSetAttribute(k_coarse_dsmem<float, 2>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -336,28 +331,41 @@ int coarse_cluster_size() {
     cudaFuncSetAttribute(k_coarse_dsmem2<double>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     cudaGetLastError();
     for (int cs : {16, 8}) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(cs, 1, 1);
-    cfg.blockDim = dim3(kCoarseThreads, 1, 1);
-    cfg.dynamicSmemBytes = kCoarseSmemMax;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = cs;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    int nclusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&nclusters, k_coarse_dsmem<float, 2>, &cfg) == cudaSuccess && nclusters >= 1) {
-        g_fit_size3 = float_unprepared ? 1 : cs;
-        g_cluster_size = cs;
-        return cs;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(cs, 1, 1);
+        cfg.blockDim = dim3(kCoarseThreads, 1, 1);
+        cfg.dynamicSmemBytes = kCoarseSmemMax;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = cs;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int nclusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&nclusters, k_coarse_dsmem<float, 2>, &cfg) == cudaSuccess && nclusters >= 1)
+            return cs;
+        cudaGetLastError();
     }
-    cudaGetLastError();
-    }
-    g_fit_size3 = 1;
-    g_cluster_size = 1;
     return 1;
+}
+
+// Asked once per device, whichever thread comes first.
+int coarse_cluster_size() {
+    constexpr int kMaxDev = 64;
+    static std::atomic<int> held[kMaxDev];
+    static std::mutex mu;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) {
+        cudaGetLastError();
+        return 1;
+    }
+    int cs = held[dev].load(std::memory_order_acquire);
+    if (cs) return cs;
+    std::lock_guard<std::mutex> g(mu);
+    cs = held[dev].load(std::memory_order_relaxed);
+    if (!cs) held[dev].store(cs = query_cluster_size(), std::memory_order_release);
+    return cs;
 }
 
 template <typename T>
@@ -369,14 +377,15 @@ bool coarse_cluster_ok(const GridDesc& g, int cs) {
     return sp.smem <= kCoarseSmemMax && rows * sp.S <= cta_capacity(g);
 }
 
-// In 2D the cluster's sweeps equal the separate ones bit for bit.  The 3D ones add the neighbours in
-// another order than the tile kernels, so a level that moved from one to the other would change in its
-// last digits: in a process whose first problem is complex128, where no cluster was found before the
-// query above was right, the 3D levels beyond one CTA stay with separate sweeps.
+// Whether the level runs in a cluster, by its size and precision and the device alone.  In 2D the
+// cluster's sweeps equal the separate ones bit for bit.  The 3D ones add the neighbours in another order
+// than the tile kernels, and pay only where one CTA could hold the level: HSS step with the cluster / with
+// separate sweeps, us, 17^3 44.2 / 51.2, 41^3 48.6 / 53.3, 65^3 68.5 / 69.8, but 73^3 (10^3 coarsest
+// nodes, the last that fits) 75.7 / 74.8, 97^3 96.9 / 96.8, 129^3 153 / 149, 161^3 246 / 233 (four
+// problems of 97^3 295 / 302, of 129^3 579 / 585).
 template <typename T>
 bool coarse_fits(const GridDesc& g) {
-    const int cs = coarse_cluster_size();
-    return coarse_cluster_ok<T>(g, g.dim == 3 ? g_fit_size3 : cs);
+    return coarse_cluster_ok<T>(g, g.dim == 3 ? 1 : coarse_cluster_size());
 }
 
 template <typename T>
