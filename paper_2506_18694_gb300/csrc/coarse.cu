@@ -71,9 +71,11 @@ constexpr int kCoarseThreads1 = 640;
 template <typename T, int K>
 __global__ void __launch_bounds__(K == 1 ? kCoarseThreads1 : kCoarseThreads)
 k_coarse_dsmem(const __grid_constant__ MArgs<T> a, int nsweeps, int per) {
-    pdl_entry();
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cg::cluster_group cl = cg::this_cluster();
+    cl.sync();  // every CTA has started before any plane is stored to another (while the previous kernel ends)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int rank = (int)cl.block_rank();
     const int prob = blockIdx.x / (int)cl.num_blocks();
     if (problem_skipped(a, prob)) return;  // uniform over the cluster: no barrier is left waiting
