@@ -480,7 +480,11 @@ __device__ __forceinline__ Cx<T> band_apply(const GsWeights<T>* wt, const vec2<T
         const GsWeights<T>& c = wt[8];
         return fma_c(c.w[3], dg, fma_c(c.w[1], hx + vy, cmul(c.w[0], ld<T>(p, 0))));
     }
-    return fma_c(k.w[3], dg, fma_c(k.w[2], vy, fma_c(k.w[1], hx, cmul(k.w[0], ld<T>(p, 0)))));
+    // (an inner node's four edge neighbours are added first here too, as the stencil kernels do: each product is
+    // rounded at the size of the centre's, and a fourth one made the W-cycle's error 3.5 % larger up to 129^2)
+    const bool in = ((d >> 16) & 15) == 8;
+    const Cx<T> e = in ? hx + vy : hx, v = in ? cx<T>(0, 0) : vy;
+    return fma_c(k.w[3], dg, fma_c(k.w[2], v, fma_c(k.w[1], e, cmul(k.w[0], ld<T>(p, 0)))));
 }
 
 // w to the neighbours' halo rows of basis vector `to`, and (after a sum) from there
