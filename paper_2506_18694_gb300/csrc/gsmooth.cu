@@ -279,7 +279,8 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_update(vec2<T>* __restrict__ 
 // Why.  A step of 5 iterations as separate kernels is 34 launches of 3 to 4 us, and in one CTA with the
 // basis in global memory it took 85 us on 65^2.  Here (GB300, complex64, 5 iterations) a step takes
 // 12 us on 9^2, 18 on 33^2, 24 on 65^2, 33 on 129^2 and 62 on 257^2; the W-cycle of 257^2 went from 2372 to
-// 712 us, of 129^2 from 1535 to 531, complex128 129^2 from 9428 to 3400.  A small level is bound by the
+// 709 us, of 129^2 from 1535 to 528, complex128 129^2 from 9428 to 3419; 16 problems of 129^2 1694 to 845, 64 of
+// 2045 to 1810, 64 of 257^2 6164 to 4500, complex128 32 of 129^2 11238 to 9785.  A small level is bound by the
 // chain of two sums an iteration (500 cycles in a block, 1350 more for the cluster barrier),
 // 257^2 by the shared-memory reads of the basis (four times an iteration).
 //
@@ -291,12 +292,10 @@ __global__ void __launch_bounds__(kGsThreads) k_gs_update(vec2<T>* __restrict__ 
 // coefficients of that pass and w before it, h^2 = ||w||^2 - ||c||^2, exact to rounding while ||c||^2 is
 // a small part of ||w||^2; else (w almost in the space already) it is summed by itself.
 //
-// Sums: a thread's and a warp's in the level precision; over the warps and the CTAs as pairs of
-// a sum and its rounding error (complex64), in a fixed order.
-#ifndef GSNT
-#define GSNT 1024
-#define GSKN 5
-#endif
+// Sums: a thread's and a warp's in the level precision; over the warps and the CTAs, in a fixed order, as
+// pairs of a sum and its rounding error in complex64 (error-free addition, Knuth's TwoSum).  A coefficient of
+// H and the norm are formed from the pairs and rounded once, as the separate kernels form them in FP64,
+// which this part does 64 times slower.
 template <typename T> struct GsCfg;  // threads a CTA at most
 template <> struct GsCfg<float> {
     static constexpr int kThreads = 1024;
@@ -318,6 +317,10 @@ template <> struct Sum<float> {
     __device__ static Sum of(float v) { return Sum{v, 0.0f}; }
     // (an infinite or NaN sum makes its rounding error NaN: the sum alone counts then)
     __device__ float value() const { return lo == lo ? hi + lo : hi; }
+    __device__ float rest(float v) const {  // what v = value() leaves out
+        const float r = __fadd_rn(__fsub_rn(hi, v), lo);
+        return r == r ? r : 0.0f;
+    }
     __device__ Sum plus_lane(int o) const {
         const float h2 = __shfl_xor_sync(0xffffffffu, hi, o), l2 = __shfl_xor_sync(0xffffffffu, lo, o);
         const float t = __fadd_rn(hi, h2), bb = __fsub_rn(t, hi);
@@ -329,8 +332,18 @@ template <> struct Sum<double> {
     double hi;
     __device__ static Sum of(double v) { return Sum{v}; }
     __device__ double value() const { return hi; }
+    __device__ double rest(double) const { return 0.0; }
     __device__ Sum plus_lane(int o) const { return Sum{hi + __shfl_xor_sync(0xffffffffu, hi, o)}; }
 };
+
+// (a + la) + (b + lb) rounded once, la and lb small beside a and b
+__device__ __forceinline__ float add_pairs(float a, float la, float b, float lb) {
+    const float t = __fadd_rn(a, b), bb = __fsub_rn(t, a);
+    const float err = __fadd_rn(__fsub_rn(a, __fsub_rn(t, bb)), __fsub_rn(b, bb));
+    const float r = __fadd_rn(t, __fadd_rn(err, __fadd_rn(la, lb)));
+    return r == r ? r : t;
+}
+__device__ __forceinline__ double add_pairs(double a, double, double b, double) { return a + b; }
 
 // Weights of a node's kind (boundary class 0..7, 8 inner): centre, x, y and diagonal neighbours,
 // omega D^{-1}.
@@ -343,8 +356,9 @@ template <typename T> struct GsShared {
     GsWeights<T> wt[9];
     T red[32][kGsScal + 2];  // sums of the warps (a group of sums may end beyond the last vector's)
     Sum<T> part[2][kGsClusterMax][kGsScal];
-    T H[kGsMaxIts][2][kGsScal];  // the sums of column j: both passes' coefficients; ||w||^2
-    T beta2, tmp, h[kGsMaxIts];
+    // column j at j & 1: its sums (both passes' coefficients; ||w||^2), and what rounding left out of them
+    T H[2][2][kGsScal], L[2][2][kGsScal];
+    T beta2, tmp, low, h[kGsMaxIts];
     Cx<T> R[kGsMaxIts][kGsMaxIts];
     Cx<T> g[kGsMaxVec], sn[kGsMaxIts], ys[kGsMaxIts];
     T cs[kGsMaxIts];
@@ -382,13 +396,17 @@ __device__ __forceinline__ void warp_sums(T* v, T* red) {
     if ((lane & (32 / S - 1)) == 0) red[lane / (32 / S)] = v[0];
 }
 
-// Column `col` of H, from both passes' sums and the norm h below its diagonal: the previous
-// rotations, then the one that zeroes h; the right side g with it.
+// Column `col` of H, from both passes' sums (added by the lanes of a warp) and the norm h below its
+// diagonal: the previous rotations, then the one that zeroes h; the right side g with it (by its lane 0).
 template <typename T>
 __device__ __forceinline__ void rotate_column(GsShared<T>& s, int col) {
-    auto H = [&](int i) {
-        return cx<T>(s.H[col][0][2 * i] + s.H[col][1][2 * i], s.H[col][0][2 * i + 1] + s.H[col][1][2 * i + 1]);
-    };
+    const int lane = threadIdx.x & 31;
+    T(*Hc)[kGsScal] = s.H[col & 1];
+    const T(*Lc)[kGsScal] = s.L[col & 1];
+    if (lane < 2 * (col + 1)) Hc[0][lane] = add_pairs(Hc[0][lane], Lc[0][lane], Hc[1][lane], Lc[1][lane]);
+    __syncwarp();
+    if (lane) return;
+    auto H = [&](int i) { return cx<T>(Hc[0][2 * i], Hc[0][2 * i + 1]); };
     Cx<T> a = H(0);
     for (int i = 0; i < col; ++i) {
         Cx<T> q = H(i + 1);
@@ -436,10 +454,11 @@ __device__ __forceinline__ void back_substitute(GsShared<T>& s, int its) {
     }
 }
 
-// The warps' sums red[.][0..ns) over the cluster into out, the same in every CTA.  rot >= 0: meanwhile
-// the last warp reduces column rot by rotations.
+// The warps' sums red[.][0..ns) over the cluster into out, and what rounding left out of them into low, the
+// same in every CTA.  rot >= 0: while the cluster meets, the last warp reduces column rot by rotations
+// (before its arrival the W-cycle of 257^2 took 727 us instead of 709).
 template <typename T>
-__device__ __forceinline__ void cluster_sums(GsCtx<T>& x, int ns, T* out, int rot = -1) {
+__device__ __forceinline__ void cluster_sums(GsCtx<T>& x, int ns, T* out, T* low, int rot = -1) {
     const int nw = blockDim.x >> 5, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     GsShared<T>& sh = *x.sh;
     __syncthreads();
@@ -449,19 +468,24 @@ __device__ __forceinline__ void cluster_sums(GsCtx<T>& x, int ns, T* out, int ro
 #pragma unroll
         for (int o = 16; o >= 1; o >>= 1) t = t.plus_lane(o);  // (every lane ends with the sum)
         if (x.cs == 1) {
-            if (lane == 0) out[q] = t.value();
+            if (lane == 0) low[q] = t.rest(out[q] = t.value());
         } else if (lane < x.cs) {
             *cg::this_cluster().map_shared_rank(&part[x.rank][q], lane) = t;
         }
     }
-    if (rot >= 0 && threadIdx.x == blockDim.x - 32) rotate_column<T>(sh, rot);
-    if (x.cs > 1) {
+    const bool rotates = rot >= 0 && threadIdx.x >= blockDim.x - 32;
+    if (x.cs == 1) {
+        if (rotates) rotate_column<T>(sh, rot);
+    } else {
         __syncwarp();
-        cg::this_cluster().sync();
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        if (rotates) rotate_column<T>(sh, rot);
+        __syncwarp();
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
         for (int q = wid; q < ns; q += nw) {
             Sum<T> t = lane < x.cs ? part[lane][q] : Sum<T>::of(T(0));
             for (int o = x.cs >> 1; o >= 1; o >>= 1) t = t.plus_lane(o);
-            if (lane == 0) out[q] = t.value();
+            if (lane == 0) low[q] = t.rest(out[q] = t.value());
         }
         ++x.phase;
     }
@@ -525,7 +549,7 @@ template <typename T, int KN>
 __device__ __forceinline__ T orthogonalise(GsCtx<T>& x, const unsigned* d, Cx<T>* w, int nv, bool more) {
     constexpr int kGroup = 4;
     GsShared<T>& sh = *x.sh;
-    T(*H)[kGsScal] = sh.H[nv - 1];
+    T(*H)[kGsScal] = sh.H[(nv - 1) & 1], (*L)[kGsScal] = sh.L[(nv - 1) & 1];
     if (more) send_rows<T, KN>(x, d, w, nv);
     T sq = T(0);
 #pragma unroll 1
@@ -550,7 +574,7 @@ __device__ __forceinline__ T orthogonalise(GsCtx<T>& x, const unsigned* d, Cx<T>
             warp_sums<T, 2 * kGroup>(acc, &sh.red[threadIdx.x >> 5][2 * i0]);
         }
         if (pass) norm_share<T, KN>(x, d, w, 2 * nv);
-        cluster_sums<T>(x, 2 * nv + pass, H[pass], pass ? -1 : nv - 2);
+        cluster_sums<T>(x, 2 * nv + pass, H[pass], L[pass], pass ? -1 : nv - 2);
         if (!pass && more) take_rows<T, KN>(x, d, w, nv);
         v0 = x.V;
 #pragma unroll 1
@@ -571,9 +595,9 @@ __device__ __forceinline__ T orthogonalise(GsCtx<T>& x, const unsigned* d, Cx<T>
         }
     }
     const T before = H[1][2 * nv];
-    if (sq <= before * T(1.0 / 64)) return before - sq;
+    if (sq <= before * T(1.0 / 64)) return before + (L[1][2 * nv] - sq);
     norm_share<T, KN>(x, d, w, 0);
-    cluster_sums<T>(x, 1, &sh.tmp);
+    cluster_sums<T>(x, 1, &sh.tmp, &sh.low);
     return sh.tmp;
 }
 
@@ -713,7 +737,7 @@ __global__ void __launch_bounds__(GsCfg<T>::kThreads) k_gs_step(const __grid_con
         } else {
             send_rows<T, KN>(X, d, w, 0);
             norm_share<T, KN>(X, d, w, 0);
-            cluster_sums<T>(X, 1, &sh.beta2);
+            cluster_sums<T>(X, 1, &sh.beta2, &sh.low);
             take_rows<T, KN>(X, d, w, 0);
             h2 = sh.beta2;
         }
@@ -736,7 +760,7 @@ __global__ void __launch_bounds__(GsCfg<T>::kThreads) k_gs_step(const __grid_con
 #pragma unroll
     for (int k = 0; k < KN; ++k) w[k] = !xzero && (d[k] & kGsIn) ? ld<T>(xb, tid + k * NT) : cx<T>(0, 0);
     if (tid < 32) {
-        if (tid == 0) rotate_column<T>(sh, its - 1);
+        rotate_column<T>(sh, its - 1);
         __syncwarp();
         back_substitute<T>(sh, its);
     }
