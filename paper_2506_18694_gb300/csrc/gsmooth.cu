@@ -14,6 +14,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 
 #include "internal.h"
@@ -799,23 +800,28 @@ int gs_cluster_of() {
     return 1;
 }
 
-// Configure k_gs_step<T> and find the largest cluster of it that the device holds (once per device).
+// Configure k_gs_step<T> and find the largest cluster of it that the device holds (once per device; asked
+// for at every smoothing step, so the answer is read without the lock).
 template <typename T>
 int gs_cluster_max() {
     constexpr int kMaxDev = 64;
     static std::mutex mu;
-    static int held[kMaxDev];  // 0: not looked at yet, -1: not available
+    static std::atomic<int> held[kMaxDev];  // 0: not looked at yet, -1: not available
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) {
         cudaGetLastError();
         return -1;
     }
+    int cs = held[dev].load(std::memory_order_acquire);
+    if (cs) return cs;
     std::lock_guard<std::mutex> g(mu);
-    if (!held[dev]) {
-        held[dev] = std::min({gs_cluster_of<T, 1>(), gs_cluster_of<T, 2>(), gs_cluster_of<T, 5>()});
+    cs = held[dev].load(std::memory_order_relaxed);
+    if (!cs) {
+        cs = std::min({gs_cluster_of<T, 1>(), gs_cluster_of<T, 2>(), gs_cluster_of<T, 5>()});
         cudaGetLastError();
+        held[dev].store(cs, std::memory_order_release);
     }
-    return held[dev];
+    return cs;
 }
 
 // nodes of the largest band with its halo rows

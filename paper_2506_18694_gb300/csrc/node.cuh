@@ -1,5 +1,5 @@
-// Per-node evaluation of a Q1 operator row from the 3^dim neighbourhood (generic
-// one-thread-per-node form, used by the 3D kernels and the small-grid solvers).
+// Per-node evaluation of a 3D Q1 operator row from the 3^3 neighbourhood (one thread per node, used by the 3D
+// coarsest level's cluster kernel).
 #pragma once
 
 #include "common.cuh"
@@ -11,51 +11,8 @@ template <typename T> struct NodeResult {
     Cx<T> d;   // diagonal entry of op at the node
 };
 
-// (op x) and diag(op) at node (i,j) of a 2D grid; rows rx, ry precomputed.
+// (op x) and diag(op) at node (i,j,l) of a 3D grid; rows rx, ry, rz precomputed.
 // x is indexed by global node number minus `off` (a slab window of the grid).
-template <typename T, bool NEED_AX>
-__device__ __forceinline__ NodeResult<T> node2(const vec2<T>* __restrict__ x, int nn, int i, int j,
-                                               const Row1<T>& rx, const Row1<T>& ry,
-                                               const OpCoef<T>& op, long long off = 0) {
-    NodeResult<T> r;
-    const T fxw = rx.face ? ry.mc : T(0);
-    const T fyw = ry.face ? rx.mc : T(0);
-    const T dr = op.cK * (rx.kc * ry.mc + rx.mc * ry.kc);
-    const T dm = rx.mc * ry.mc;
-    const T dg = fxw + fyw;
-    r.d = cx<T>(dr + op.cM.re * dm + op.cG.re * dg, op.cM.im * dm + op.cG.im * dg);
-    if (!NEED_AX) {
-        r.ax = cx<T>(0, 0);
-        return r;
-    }
-    const int ia[3] = {rx.lo, i, rx.hi};
-    const int jb[3] = {ry.lo, j, ry.hi};
-    const T myw[3] = {ry.ml, ry.mc, ry.mr};
-    const T kyw[3] = {ry.kl, ry.kc, ry.kr};
-    Cx<T> Mx = cx<T>(0, 0), Kx = cx<T>(0, 0), Fx = cx<T>(0, 0), mxc = cx<T>(0, 0);
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-        const long long row = (long long)jb[b] * nn - off;
-        const Cx<T> v0 = ld<T>(x, row + ia[0]);
-        const Cx<T> v1 = ld<T>(x, row + ia[1]);
-        const Cx<T> v2 = ld<T>(x, row + ia[2]);
-        Cx<T> mx = fma_r(rx.mr, v2, fma_r(rx.mc, v1, rx.ml * v0));
-        Cx<T> kx = fma_r(rx.kr, v2, fma_r(rx.kc, v1, rx.kl * v0));
-        Mx = fma_r(myw[b], mx, Mx);
-        Kx = fma_r(myw[b], kx, fma_r(kyw[b], mx, Kx));
-        Fx = fma_r(myw[b], v1, Fx);
-        if (b == 1) mxc = mx;
-    }
-    Cx<T> F = rx.face ? Fx : cx<T>(0, 0);
-    if (ry.face) F = F + mxc;
-    Cx<T> ax = op.cK * Kx;
-    ax = fma_c(op.cM, Mx, ax);
-    ax = fma_c(op.cG, F, ax);
-    r.ax = ax;
-    return r;
-}
-
-// (op x) and diag(op) at node (i,j,l) of a 3D grid.
 template <typename T, bool NEED_AX>
 __device__ __forceinline__ NodeResult<T> node3(const vec2<T>* __restrict__ x, int nn, int i, int j,
                                                int l, const Row1<T>& rx, const Row1<T>& ry,

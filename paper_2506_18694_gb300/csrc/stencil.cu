@@ -43,7 +43,7 @@ __device__ __forceinline__ bool node_masked(const GridDesc& g, int i, int j, int
 // ---------------------------------------------------------------- restriction
 // Full weighting R = P^T: coarse node I gathers fine nodes 2I + a, a in {-1,0,1}^dim,
 // with weight prod (a == 0 ? 1 : 1/2) (the transpose of bi/trilinear interpolation).
-// grid.z = planes x problems (3D) or problems (2D).
+// grid.z = problems.  2D.
 template <typename T>
 __global__ void __launch_bounds__(256) k_restrict(GridDesc gc, const vec2<T>* __restrict__ rf,
                                                   vec2<T>* __restrict__ rc, Batch bt) {
@@ -131,42 +131,34 @@ cudaError_t launch_restrict(const GridDesc& gc, const vec2<T>* rf, vec2<T>* rc, 
 
 // ---------------------------------------------------------------- prolongation
 // x_f += P e_c: fine node i takes coarse node i/2 (even i) or the mean of (i-1)/2 and
-// (i+1)/2 (odd i) along each axis (bi/trilinear interpolation of the coarse Q1 field).
+// (i+1)/2 (odd i) along each axis (bi/trilinear interpolation of the coarse Q1 field).  2D.
 template <typename T>
 __global__ void __launch_bounds__(256) k_prolong(GridDesc gf, const vec2<T>* __restrict__ ec,
                                                  vec2<T>* __restrict__ x, Batch bt) {
     pdl_entry();
-    const bool d3 = gf.dim == 3;
-    const int planes = d3 ? gf.nn : 1;
-    const int b = blockIdx.z / planes;
-    const int l = blockIdx.z - b * planes;
+    const int b = blockIdx.z;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
     if (i > gf.n || j > gf.n || batch_skipped(bt, b)) return;
     x += (long long)b * bt.bs;
     ec += (long long)b * bt.bsc;
-    const long long p = d3 ? ((long long)l * gf.nn + j) * gf.nn + i : (long long)j * gf.nn + i;
-    if (node_masked(gf, i, j, l)) {
+    const long long p = (long long)j * gf.nn + i;
+    if (node_masked(gf, i, j, 0)) {
         st<T>(x, p, cx<T>(0, 0));
         return;
     }
     const int nc = gf.n / 2, nnc = nc + 1;
-    const int I0 = i >> 1, J0 = j >> 1, L0 = l >> 1;
-    const int ni = (i & 1) ? 2 : 1, nj = (j & 1) ? 2 : 1, nl = (d3 && (l & 1)) ? 2 : 1;
-    const T wi = (i & 1) ? T(0.5) : T(1), wj = (j & 1) ? T(0.5) : T(1),
-            wl = (d3 && (l & 1)) ? T(0.5) : T(1);
+    const int I0 = i >> 1, J0 = j >> 1;
+    const int ni = (i & 1) ? 2 : 1, nj = (j & 1) ? 2 : 1;
+    const T wi = (i & 1) ? T(0.5) : T(1), wj = (j & 1) ? T(0.5) : T(1);
     // coarse Dirichlet nodes carry no basis function: their entries are never read
     auto coarse_dir = [&](int I, int lo, int hi) { return (I == 0 && lo) || (I == nc && hi); };
     Cx<T> e = cx<T>(0, 0);
-    for (int c = 0; c < nl; ++c) {
-        if (d3 && coarse_dir(L0 + c, gf.dir[4], gf.dir[5])) continue;
-        for (int bb = 0; bb < nj; ++bb) {
-            if (coarse_dir(J0 + bb, gf.dir[2], gf.dir[3])) continue;
-            for (int a = 0; a < ni; ++a) {
-                if (coarse_dir(I0 + a, gf.dir[0], gf.dir[1])) continue;
-                const long long q = ((long long)(d3 ? L0 + c : 0) * nnc + (J0 + bb)) * nnc + (I0 + a);
-                e = fma_r(wi * wj * wl, ld<T>(ec, q), e);
-            }
+    for (int bb = 0; bb < nj; ++bb) {
+        if (coarse_dir(J0 + bb, gf.dir[2], gf.dir[3])) continue;
+        for (int a = 0; a < ni; ++a) {
+            if (coarse_dir(I0 + a, gf.dir[0], gf.dir[1])) continue;
+            e = fma_r(wi * wj, ld<T>(ec, (long long)(J0 + bb) * nnc + (I0 + a)), e);
         }
     }
     st<T>(x, p, ld<T>(x, p) + e);
@@ -175,8 +167,8 @@ __global__ void __launch_bounds__(256) k_prolong(GridDesc gf, const vec2<T>* __r
 // 3D: a thread takes coarse node (I, J, L) and the up to eight fine nodes (2I + a, 2J + b, 2L + c), so
 // that the coarse values it needs are read once; nodes are numbered through the plane (257^3 55 -> 52 us,
 // 129^3 11.7 -> 10.8).  Bound by the L1 pipe: every access steps by 16 bytes; one fine column per thread,
-// whole rows at a time, took 60 us on 257^3.  The terms of a node are added in k_prolong's order
-// (z, then y, then x), so the results are the same bit for bit.
+// whole rows at a time, took 60 us on 257^3.  The terms of a node are added by z, then y,
+// then x.
 template <typename T>
 __global__ void __launch_bounds__(256) k_prolong3(GridDesc gf, const vec2<T>* __restrict__ ec, vec2<T>* __restrict__ x,
                                                   Batch bt) {
@@ -236,7 +228,7 @@ cudaError_t launch_prolong(const GridDesc& gf, const vec2<T>* ec, vec2<T>* x, co
         return klaunch(k_prolong3<T>, dim3((nnc * nnc + 255) / 256, 1, nnc * bt.nb), dim3(256), 0, s, 1, gf, ec, x, bt);
     }
     dim3 blk(32, 8, 1);
-    dim3 grd((gf.nn + 31) / 32, (gf.nn + 7) / 8, (gf.dim == 3 ? gf.nn : 1) * bt.nb);
+    dim3 grd((gf.nn + 31) / 32, (gf.nn + 7) / 8, bt.nb);
     return klaunch(k_prolong<T>, grd, blk, 0, s, 1, gf, ec, x, bt);
 }
 
