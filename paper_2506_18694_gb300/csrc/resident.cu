@@ -5,8 +5,8 @@
 // Why.  On grids of a few hundred nodes per side a V(2,2) cycle as separate kernels is a chain
 // of 2L - 1 launches of 3-10 us each, bound by launch and tile latency, not by work.  Here a
 // pass over a level is a loop over shared memory and its end a halo exchange.  Measured (GB300, us
-// per V-cycle of the HSS loop, 4 levels; separate kernels / resident): complex64 17^2 35 / 9.4, 65^2
-// 36 / 15, 129^2 32 / 18, 257^2 35 / 30; complex128 33^2 136 / 34, 65^2 136 / 53.  A pass is bound by
+// per V-cycle of the HSS loop, 4 levels; separate kernels / resident): complex64 17^2 35 / 10, 65^2
+// 36 / 15.6, 129^2 32 / 19, 257^2 35 / 30; complex128 33^2 136 / 35, 65^2 136 / 55.  A pass is bound by
 // the latency of one dependent chain of about 330 cycles, plus about 500 for an exchange.
 //
 // Layout.  CTA r of the cluster owns rows f(r) .. f(r + 1) - 1 of level 0, f(r) = floor(r nn / cs),
@@ -31,8 +31,9 @@
 //
 // Every wait is bounded (spin_limit polls): a CTA that gives up skips the rest of its passes, but not
 // the cluster barriers; its neighbours' waits run out in turn, and the launch ends with the status
-// recorded and a result of NaN.  That a wait ran out is read by every thread behind the pass's block barrier, from a word that
-// is not written again before the next one, so the whole CTA gives up at the same pass.  What others
+// recorded and a result of NaN.  That a wait ran out is read by every thread behind the pass's block barrier,
+// from a word that is not written again before the next one, so the whole CTA gives up at the same pass
+// (a barrier that carries it itself, __syncthreads_or, made a cycle 1 to 3 % slower).  What others
 // sent to a CTA that gave up is still on its way when the passes end: the CTAs of such a cluster tell
 // one another how many passes and copies they sent, and each waits for its own (give_up).
 //
@@ -500,8 +501,10 @@ __device__ __noinline__ int restrict_pass(Res S, int lvl, int copies) {
     vec2<T>* const sm = vecs<T>();
     const Push ps = push_rows<T>(S, M, M.A);
     pass_begin<T>(S, M);
-    if (spread && threadIdx.x == 0)
+    if (spread && threadIdx.x == 0) {
+        hd.copies = copies + 1;
         bar_expect(saddr(&hd.mbr[copies & 1]), (unsigned)((M.nn - M.bulkn) * M.W * sizeof(vec2<T>)));
+    }
     const uint2* dw = reinterpret_cast<const uint2*>(words<T>() + M.r0);
     for (int it = threadIdx.x; it < M.restricted; it += kResThreads) {
         // x: offset of fine node (2I, 2J - 1) in A, and of coarse node (I, J) in an iterate << 16
@@ -623,10 +626,11 @@ __device__ __forceinline__ int peer(const int* p, int rank) {
 // will): a CTA that gave up waits for what is still on its way to it, so that none of it arrives after the
 // CTA has left.  Of the halo rows that is its last pass's, if the neighbour sent them, and those of one
 // pass more, in which the neighbour gave up for want of our rows (hence its row_bytes); of the right
-// sides (`copies` sent here so far, level lr) the last one's from the CTAs that sent it, and the next one's.
+// sides (of level lr) the last one's from the CTAs that sent it, and the next one's.
 template <typename T>
-__device__ __noinline__ void give_up(const Res S, int copies, int lr) {
+__device__ __noinline__ void give_up(const Res S, int lr) {
     Head<T>& hd = head<T>();
+    const int copies = hd.copies;
     constexpr unsigned long long kDrain = 4194304;  // (microseconds are enough)
     const int r = S.round & ~kDead;
     if ((threadIdx.x == 0 && S.rank > 0) || (threadIdx.x == 32 && S.rank + 1 < S.cs)) {
@@ -840,7 +844,7 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident2(const __grid_const
         for (int q = 0; q < 2; ++q)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(saddr(&hd.mbr[q])) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        hd.gave_up[0] = hd.gave_up[1] = hd.gave_up[2] = hd.any = 0;
+        hd.gave_up[0] = hd.gave_up[1] = hd.gave_up[2] = hd.any = hd.copies = 0;
     } else if (threadIdx.x == 32) {
         const int nn0 = a.lv[0].nn;
         int f0 = S.rank * nn0 / a.cs, f1 = (S.rank + 1) * nn0 / a.cs, fu = S.rank > 0 ? (S.rank - 1) * nn0 / a.cs : 0;
@@ -884,7 +888,6 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident2(const __grid_const
     if (copies) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 
     const int steps = HSS ? a.nhss[prob] : 1;
-    int sent = 0;  // right sides sent to the other CTAs
     for (int it = 0; it < steps; ++it) {
         if (HSS) {
             if (!keep) {
@@ -900,7 +903,6 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident2(const __grid_const
         }
         for (int l = 0; l < Lc - 1; ++l) {
             S.round = passes<T, P_SWEEP, P_RESID>(S, l, l, hd.lv[l].A, hd.lv[l].B, hd.lv[l].b);
-            if (!S.dead() && l + 1 == a.dist) sent = it + 1;
             S.round = restrict_pass<T>(S, l, it);
             if (copies && l + 1 == a.dist)
                 passes<T, P_FIRST, -1>(S, l + 1, l + 1, hd.lv[l + 1].A, hd.lv[l + 1].A, hd.lv[l + 1].b);
@@ -928,14 +930,13 @@ __global__ void __launch_bounds__(kResThreads, 1) k_resident2(const __grid_const
     if (a.cs == 1) return;
     if (threadIdx.x == 0) {
         hd.rounds = S.round & ~kDead;
-        hd.copies = sent;
         if (S.dead()) *a.status = HSS ? kLoopTimeout : kCycleTimeout;
     }
     if (S.dead() && (int)threadIdx.x < S.cs)
         asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote(saddr(&hd.any), threadIdx.x)), "r"(1) : "memory");
     cg::this_cluster().sync();  // nobody leaves while another may still send to it
     if (hd.any) {
-        if (S.dead()) give_up<T>(S, sent, copies ? a.dist : 0);
+        if (S.dead()) give_up<T>(S, copies ? a.dist : 0);
         // no half-finished result: a single cycle's caller is told only by its next blocking call
         for (int q = threadIdx.x; q < L0.R * nn0; q += kResThreads) write(base + q, cx<T>(T(NAN), T(NAN)));
         __syncthreads();
@@ -1075,8 +1076,11 @@ bool resident_plan(ResArgs<T>* P, const GridDesc* lv, int levels, int nb, bool h
     }
     P->nb = nb;
     for (int q = 0; q < 4; ++q) P->dir[q] = lv[0].dir[q];
-    // the largest clusters (a problem's cycle is shortest with them) that the device holds at once:
-    // a batch in several waves of clusters is slower than the separate kernels over all its problems
+    // the largest clusters (a problem's cycle is shortest with them) that the device holds at once: a batch in
+    // several waves of clusters would be slower than the separate kernels over all its problems.  HSS step of a
+    // batch, us, here / separate: complex64 65^2 8 problems (16 CTAs) 15.7 / 45, 32 (4) 16.9 / 51, 64 (2)
+    // 19.7 / 60, 152 (1) 20.6 / 89; 97^2 76 (2) 28 / 84; 129^2 9 (8) 22 / 47, 36 (4) 28 / 77; 257^2 7 (16) 30 / 56;
+    // complex128 33^2 128 (1) 98 / 425, 65^2 64 (2) 180 / 459, 97^2 32 (4) 206 / 417, 129^2 8 (8) 186 / 279
     for (int q = 0; q < 4; ++q)
         if (active[q] >= nb && plan_for<T>(P, lv, levels, hss, 16 >> q)) return true;
     return nb <= num_sms() && plan_for<T>(P, lv, levels, hss, 1);

@@ -1125,8 +1125,9 @@ hh::ResArgs<T>* resident(hh_problem* p, bool hss) {
         H.res_state[hss] = -1;
         hh::ResArgs<T> P{};
         // measured against the separate kernels (a V-cycle of the HSS loop / alone, us, 4 levels):
-        // complex64 17^2 9 / 17 against 35 / 41, 129^2 18 / 28 against 32 / 41, 257^2 30 / 42 against
-        // 35 / 43; complex128 33^2 34 / 42 against 136 / 128, 129^2 112 / 121 against 129 / 124
+        // complex64 17^2 11 / 19 against 34 / 35, 129^2 20 / 31 against 36 / 39, 161^2 21 / 32 against 35 / 40,
+        // 257^2 30 / - against 36 / 39; complex128 33^2 35 / 44 against 134 / 128, 65^2 55 / 60 against
+        // 127 / 133, 129^2 113 / - against 140 / 129 (batches: resident_plan)
         const long long most = sizeof(T) == 4 ? (hss ? 67000 : 40000) : (hss ? 17000 : 5000);
         if (resident_options(p) && p->lv[0].N <= most &&
             hh::resident_plan<T>(&P, p->lv.data(), p->o.levels, p->nb, hss)) {
