@@ -85,7 +85,7 @@ __device__ __forceinline__ void rr_pass(const MArgs<T>& a, int strips, int chunk
         const int b = BATCH ? t / per : 0;
         if (BATCH && loop_skipped(a, b, it)) continue;
         const int r = t - b * per;
-        rr_tile<T, MODE, 1, BATCH>(a, b, r % strips, r / strips);
+        rr_tile<T, MODE, 1, BATCH, true>(a, b, r % strips, r / strips);
     }
 }
 
@@ -101,7 +101,7 @@ __device__ __forceinline__ void f_pass(const MArgs<T>& a, int strips, int chunks
         const PCoef<T>& c = BATCH ? a.pc[b] : a.c0;
         const PCoef<T>& cl = BATCH ? a.pc2[b] : a.c02;
         const VPtrs<T> v = problem_ptrs(a, b, false);
-        tilef<T, M_PROLONG_JACOBI2, 2>(a, c, cl, v, r % strips, r / strips);
+        tilef<T, M_PROLONG_JACOBI2, 2, true>(a, c, cl, v, r % strips, r / strips);
     }
 }
 

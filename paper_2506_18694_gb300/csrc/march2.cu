@@ -178,7 +178,7 @@ __device__ __forceinline__ void tile_compute(const MArgs<T>& a, const PCoef<T>& 
     }
 }
 
-// whether tile (strip, cy) takes the INNER form
+// whether tile (strip, cy) takes the INNER form where a kernel has both
 template <typename T, int MODE, int ROWS>
 __device__ __forceinline__ bool tile_in(const MArgs<T>& a, int strip, int cy) {
     using TL = Tile2<T, MODE, ROWS>;
@@ -199,7 +199,7 @@ __device__ __forceinline__ void tile_compute_any(const MArgs<T>& a, const PCoef<
 }
 
 // grid (strips of 28 columns, ceil(chunks / 4), problems)
-template <typename T, int MODE, int ROWS, bool BATCH>
+template <typename T, int MODE, int ROWS, bool BATCH, bool SPLIT>
 __global__ void __launch_bounds__(128) k_march2f(const __grid_constant__ MArgs<T> a, int chunks) {
     pdl_entry();
     const int b = BATCH ? (int)blockIdx.z : 0;
@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(128) k_march2f(const __grid_constant__ MArgs<T
     const PCoef<T>& c = BATCH ? a.pc[b] : a.c0;
     const PCoef<T>& cl = BATCH ? a.pc2[b] : a.c02;
     const VPtrs<T> v = problem_ptrs(a, b, false);
-    tilef<T, MODE, ROWS>(a, c, cl, v, blockIdx.x, cy);
+    tilef<T, MODE, ROWS, SPLIT>(a, c, cl, v, blockIdx.x, cy);
 }
 
 template <typename T, int MODE>
@@ -223,17 +223,19 @@ static cudaError_t gof(MArgs<T> a, cudaStream_t s) {
     const int chunks = (a.g.nn + rows - 1) / rows;
     const dim3 grd((unsigned)strips, (unsigned)((chunks + 3) / 4), (unsigned)a.nb);
     if (a.pc) {
-        if (rows == 4) return klaunch(k_march2f<T, MODE, 4, true>, grd, dim3(128), 0, s, 1, a, chunks);
-        return klaunch(k_march2f<T, MODE, 2, true>, grd, dim3(128), 0, s, 1, a, chunks);
+        if (rows == 4) return klaunch(k_march2f<T, MODE, 4, true, true>, grd, dim3(128), 0, s, 1, a, chunks);
+        if (a.split) return klaunch(k_march2f<T, MODE, 2, true, true>, grd, dim3(128), 0, s, 1, a, chunks);
+        return klaunch(k_march2f<T, MODE, 2, true, false>, grd, dim3(128), 0, s, 1, a, chunks);
     }
     if (a.nb != 1) return cudaErrorInvalidValue;
-    if (rows == 4) return klaunch(k_march2f<T, MODE, 4, false>, grd, dim3(128), 0, s, 1, a, chunks);
-    return klaunch(k_march2f<T, MODE, 2, false>, grd, dim3(128), 0, s, 1, a, chunks);
+    if (rows == 4) return klaunch(k_march2f<T, MODE, 4, false, true>, grd, dim3(128), 0, s, 1, a, chunks);
+    if (a.split) return klaunch(k_march2f<T, MODE, 2, false, true>, grd, dim3(128), 0, s, 1, a, chunks);
+    return klaunch(k_march2f<T, MODE, 2, false, false>, grd, dim3(128), 0, s, 1, a, chunks);
 }
 
 // One tile per warp; grid (strips, ceil(chunks / 4), problems).  BATCH = false: a batch of
 // one, coefficients from the kernel parameters and no activity flags.
-template <typename T, int MODE, int ROWS, bool BATCH>
+template <typename T, int MODE, int ROWS, bool BATCH, bool SPLIT>
 __global__ void __launch_bounds__(128) k_march2(const __grid_constant__ MArgs<T> a, int chunks) {
     pdl_entry();
     const int b = BATCH ? (int)blockIdx.z : 0;
@@ -243,7 +245,7 @@ __global__ void __launch_bounds__(128) k_march2(const __grid_constant__ MArgs<T>
     const PCoef<T>& c = BATCH ? a.pc[b] : a.c0;
     const VPtrs<T> v = problem_ptrs(a, b, MODE == M_RESID_RESTRICT);
     Tile2<T, MODE, ROWS> tl;
-    if (tile_in<T, MODE, ROWS>(a, blockIdx.x, cy)) {
+    if (SPLIT && tile_in<T, MODE, ROWS>(a, blockIdx.x, cy)) {
         tile_load<T, MODE, ROWS, true>(a, v, blockIdx.x, cy, tl);
         tile_compute<T, MODE, ROWS, true>(a, c, v, blockIdx.x, cy, tl);
     } else {
@@ -396,7 +398,9 @@ static cudaError_t run2b(const MArgs<T>& a, int strips, int chunks, cudaStream_t
         }
     }
     dim3 grd((unsigned)strips, (unsigned)((chunks + 3) / 4), (unsigned)a.nb);
-    return klaunch(k_march2<T, MODE, ROWS, BATCH>, grd, dim3(128), 0, s, 1, a, chunks);
+    if (ROWS == 2 && !a.split)
+        return klaunch(k_march2<T, MODE, ROWS, BATCH, ROWS != 2>, grd, dim3(128), 0, s, 1, a, chunks);
+    return klaunch(k_march2<T, MODE, ROWS, BATCH, true>, grd, dim3(128), 0, s, 1, a, chunks);
 }
 
 template <typename T, int MODE, int ROWS>

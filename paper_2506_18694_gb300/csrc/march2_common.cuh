@@ -39,7 +39,8 @@ __device__ __forceinline__ bool row_void(const MArgs<T>& a, int r) {
 
 // Whether a tile of 32 columns from `left` and `rows` rows from `first` lies inside the grid, off its
 // sides (at least `off` nodes): no node of it is void, on a boundary or beside the grid, and the tile
-// functions compile without those checks (INNER).  Uniform over the warp.
+// functions compile without those checks (INNER).  Uniform over the warp.  Kernels whose grids may be small
+// (tiles of 2 rows, or 1 coarse row) exist with both forms and with the checked one alone (SPLIT).
 template <typename T>
 __device__ __forceinline__ bool tile_inner2(const MArgs<T>& a, int left, int first, int rows, int off = 1) {
     return left >= off && left + 31 <= a.g.n - off && first >= off && first + rows - 1 <= a.g.n - off;
@@ -221,12 +222,12 @@ __device__ __forceinline__ void tilef_compute(const MArgs<T>& a, const PCoef<T>&
     }
 }
 
-// One warp's tile of a fused mode.
-template <typename T, int MODE, int ROWS>
+// One warp's tile of a fused mode (SPLIT: in both forms).
+template <typename T, int MODE, int ROWS, bool SPLIT>
 __device__ __forceinline__ void tilef(const MArgs<T>& a, const PCoef<T>& c, const PCoef<T>& cl, const VPtrs<T>& v,
                                       int strip, int cy) {
     TileF<T, ROWS> tl;
-    if (tile_inner2(a, strip * 28 - 2, cy * ROWS - 2, ROWS + 4, MODE == M_PROLONG_JACOBI2 ? 2 : 1)) {
+    if (SPLIT && tile_inner2(a, strip * 28 - 2, cy * ROWS - 2, ROWS + 4, MODE == M_PROLONG_JACOBI2 ? 2 : 1)) {
         tilef_load<T, MODE, ROWS, true>(a, v, strip, cy, tl);
         tilef_compute<T, MODE, ROWS, true>(a, c, cl, v, strip, cy, tl);
     } else {
@@ -398,10 +399,10 @@ __device__ __forceinline__ void rr_tile_of(const MArgs<T>& a, int b, int strip, 
         }
     }
 }
-template <typename T, int MODE, int CR, bool BATCH>
+template <typename T, int MODE, int CR, bool BATCH, bool SPLIT>
 __device__ __forceinline__ void rr_tile(const MArgs<T>& a, int b, int strip, int cy) {
     using G = RRGeo<MODE, CR>;
-    if (tile_inner2(a, strip * G::S - G::OFF, 2 * cy * CR - 1 - G::RES0, G::NF))
+    if (SPLIT && tile_inner2(a, strip * G::S - G::OFF, 2 * cy * CR - 1 - G::RES0, G::NF))
         rr_tile_of<T, MODE, CR, BATCH, true>(a, b, strip, cy);
     else
         rr_tile_of<T, MODE, CR, BATCH, false>(a, b, strip, cy);

@@ -11,14 +11,14 @@
 namespace hh {
 
 // grid (strips, ceil(chunks / 4), problems); chunk = CR coarse rows
-template <typename T, int MODE, int CR, bool BATCH>
+template <typename T, int MODE, int CR, bool BATCH, bool SPLIT>
 __global__ void __launch_bounds__(128) k_march2rr(const __grid_constant__ MArgs<T> a, int chunks) {
     pdl_entry();
     const int b = BATCH ? (int)blockIdx.z : 0;
     const int cy = blockIdx.y * 4 + (threadIdx.x >> 5);
     if (cy >= chunks) return;
     if (BATCH && problem_skipped(a, b)) return;
-    rr_tile<T, MODE, CR, BATCH>(a, b, blockIdx.x, cy);
+    rr_tile<T, MODE, CR, BATCH, SPLIT>(a, b, blockIdx.x, cy);
 }
 
 template <typename T, int MODE>
@@ -36,12 +36,14 @@ static cudaError_t gorr(MArgs<T> a, cudaStream_t s) {
     const int chunks = (nnc + cr - 1) / cr;
     const dim3 grd((unsigned)strips, (unsigned)((chunks + 3) / 4), (unsigned)a.nb);
     if (a.pc) {
-        if (cr == 2) return klaunch(k_march2rr<T, MODE, 2, true>, grd, dim3(128), 0, s, 1, a, chunks);
-        return klaunch(k_march2rr<T, MODE, 1, true>, grd, dim3(128), 0, s, 1, a, chunks);
+        if (cr == 2) return klaunch(k_march2rr<T, MODE, 2, true, true>, grd, dim3(128), 0, s, 1, a, chunks);
+        if (a.split) return klaunch(k_march2rr<T, MODE, 1, true, true>, grd, dim3(128), 0, s, 1, a, chunks);
+        return klaunch(k_march2rr<T, MODE, 1, true, false>, grd, dim3(128), 0, s, 1, a, chunks);
     }
     if (a.nb != 1) return cudaErrorInvalidValue;
-    if (cr == 2) return klaunch(k_march2rr<T, MODE, 2, false>, grd, dim3(128), 0, s, 1, a, chunks);
-    return klaunch(k_march2rr<T, MODE, 1, false>, grd, dim3(128), 0, s, 1, a, chunks);
+    if (cr == 2) return klaunch(k_march2rr<T, MODE, 2, false, true>, grd, dim3(128), 0, s, 1, a, chunks);
+    if (a.split) return klaunch(k_march2rr<T, MODE, 1, false, true>, grd, dim3(128), 0, s, 1, a, chunks);
+    return klaunch(k_march2rr<T, MODE, 1, false, false>, grd, dim3(128), 0, s, 1, a, chunks);
 }
 
 template <typename T>

@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(128) k_pack_rr(const HssLoop2<T>* __restrict__
     const MArgs<T>& a = MODE == M_HSS_FIRST2_RR ? (it == 0 ? P.first : P.pre[0]) : P.pre[level];
     const int strips = P.pre_strips[level];
     const int r = t - starts[m];
-    rr_tile<T, MODE, 1, false>(a, 0, r % strips, r / strips);
+    rr_tile<T, MODE, 1, false, true>(a, 0, r % strips, r / strips);
 }
 
 // prolongation + two sweeps on level `level`; 4 warp tiles per CTA
@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(128) k_pack_f(const HssLoop2<T>* __restrict__ 
     const int strips = P.post_strips[level];
     const int r = t - starts[m];
     const VPtrs<T> v = problem_ptrs(a, 0, false);
-    tilef<T, M_PROLONG_JACOBI2, 2>(a, a.c0, a.c02, v, r % strips, r / strips);
+    tilef<T, M_PROLONG_JACOBI2, 2, true>(a, a.c0, a.c02, v, r % strips, r / strips);
 }
 
 // the coarsest level: one CTA per band of coarse_rows rows of one problem

@@ -459,6 +459,13 @@ struct MG {
         a.omega = omega;
         a.tile_rows = p->o.tile_rows;
         a.tile_form = p->o.tile_form;
+        // The check-free tile form saves instructions, but a cycle on a small grid waits for instruction fetches,
+        // which its code makes longer: every level's kernels take it from a finest grid of 200k nodes
+        // (complex128 55k) up.  HSS step, us, without / with: complex64 265^2 32.7 / 36.2, 401^2 35.6 / 36.9, 449^2
+        // 37.6 / 37.6, 561^2 43.3 / 41.4, 1025^2 71.2 / 62.8; 8 problems of 129^2 45.7 / 46.6, of 201^2 53.5 / 52.4;
+        // complex128 137^2 142 / 155, 201^2 163 / 169, 265^2 239 / 192.  (By level instead, both codes in one cycle
+        // cost 1 to 2 us more: 305^2 35.8.)
+        a.split = p->lv[0].N * p->nb >= (sizeof(T) == 4 ? 200000 : 55000);
         a.hss_it = p->nb == 1 ? -1 : hss_it;
         a.nhss = p->d_nhss;
         a.active = active_flags(p);
