@@ -65,7 +65,7 @@ static SlabPlan slab_plan(const GridDesc& g, int cs) {
 // from the table entry of A_L on this level (interior weights and omega D^{-1} included).
 // K nodes per thread; a sweep lasts as long as one warp's chain over them (nodes near a side take about
 // 400 instructions), so K = 1 wherever the CTA's nodes allow, with the 1D rows kept over the sweeps, and
-// the cluster is the smallest that gives each thread a node (fewer CTAs to wait for).  HSS step with the
+// the cluster is the smallest that gives each thread a node (batch_cluster_size).  HSS step with the
 // coarsest level 3^3, 5^3, 6^3, us: 48.2 -> 43.7, 51.6 -> 46.1, 52.6 -> 48.5.
 constexpr int kCoarseThreads1 = 640;
 template <typename T, int K>
@@ -416,10 +416,13 @@ template <typename T>
 static int batch_cluster_size(const GridDesc& g, int nb) {
     int cs = coarse_cluster_size();
     while (cs > 1 && (long long)nb * cs > 2LL * num_sms() && coarse_cluster_ok<T>(g, cs / 2)) cs /= 2;
-    // 3D: no more CTAs than give each thread a node (a smaller cluster's barriers cost less)
+    // 3D: no more CTAs than give each thread a node (a smaller cluster's barriers cost less).  A complex128
+    // sweep is bound by the FP64 pipe of each SM: no more than 128 nodes, a warp for each of its four parts.
+    // HSS step, us, complex128, 512 / 128 nodes / always 16 CTAs: 17^3 with two levels 253 / 144 / 144, 25^3 with
+    // three 322 / 222 / 212, four of them 343 / 251 / 313, 33^3 336 / 224 / 223, 16 of 17^3 322 / 319 / 365
     auto one_each = [&](int c) {
         const SlabPlan sp = slab_plan<T>(g, c);
-        return sp.per * sp.S <= kCoarseThreads && sp.smem <= kCoarseSmemMax;
+        return sp.per * sp.S <= (sizeof(T) == 4 ? kCoarseThreads : 128) && sp.smem <= kCoarseSmemMax;
     };
     while (g.dim == 3 && cs > 1 && one_each(cs / 2)) cs /= 2;
     return cs;
