@@ -379,7 +379,8 @@ HH_API hh_status hh_multidot_noalloc(const void* V, long long ld, int nvec, cons
  * iteration of a member is the same sequence of operations as in its own hh_solve (same kernels,
  * on the member's own stream), except that the preconditioner applications (Def. 4.1) of all
  * members that need one in the same round run together: each pass of the V-cycle is ONE launch
- * covering the tiles of every member, whatever its grid, replayed from a CUDA graph.  Members
+ * covering the tiles of every such member, whatever its grid, replayed from a CUDA graph.  A member
+ * whose HSS loop is one kernel anyway (a small grid in one cluster) runs it on its own stream.  Members
  * join (hh_pack_add) and leave (hh_pack_take) between rounds, so a finished member's slot can be
  * refilled at once while the others go on.  Each member's result equals its own hh_solve's bit
  * for bit.  Members: problems of hh_create_problem (one problem each) in 2D, primal, with
@@ -398,7 +399,8 @@ HH_API hh_status hh_pack_create(int capacity, hh_pack** out);
  * the member's slot.  HH_ERR_INVALID if p cannot be packed, the pack is full or p is in it. */
 HH_API hh_status hh_pack_add(hh_pack* k, hh_problem* p, const void* rhs, int io, double tol, void* u, int* slot);
 
-/* Run rounds (every running member advances to its next synchronisation point) until at least
+/* Run rounds (every member of the shared launches advances to its next synchronisation point, and of the
+ * members with a loop of their own each whose work is done; at least one member advances) until at least
  * one member has finished, no member is running, or max_rounds rounds (> 0) have run; done (room
  * for `capacity` ints) receives the slots of every finished member not yet taken, *ndone their
  * number. */
